@@ -1,0 +1,239 @@
+// collide64.cuh - the cell update of the FP64 form (a3 - a6), written for the fewest
+// FP64 operations.  Included by kernels.cuh after the shared helpers.
+//
+// What bounds it: a quarter of an SM (one scheduler) takes 64 cycles for an FP64
+// instruction, whatever the number of active lanes (measured, dependent or not; a
+// conversion between FP64 and FP32 costs the same), so the form is bound by its FP64
+// instruction count and not by memory: 1520 bytes a D3Q95 cell take 0.23 ns of HBM time,
+// the ~1270 FP64 operations of the pair-by-pair form 2.4 ns.  Three regroupings bring
+// D3Q95 to ~890 operations a cell:
+//   * moments shell by shell: the members of a shell share weight and |xi|^2, so their
+//     sums are formed unweighted (momentum in units of the primitive vector) and each
+//     shell is weighted once;
+//   * rho and rho - 1 folded into the shell's equilibrium coefficients, so a pair's
+//     even part is c0 + s^2 (c2 + s^2 c4) and its odd part s (c1 + s^2 c3);
+//   * s and s^2 once per primitive direction b: the pairs k b of several shells (axes
+//     2, 3, 5; diagonals 2, 3, 4; ...) share them, with the powers of k folded into the
+//     coefficients.
+//
+// The shells are dealt into kParts64 parts of nearly equal work (whole shells, so the
+// weighting is not repeated).  Every kernel sums the parts' moments in the same order,
+// ((0 + 1) + (2 + 3)), so one thread doing all parts and several warps doing some each
+// produce the same bits.
+#pragma once
+
+namespace lbm {
+
+constexpr int kParts64 = 4;
+
+// The part each shell belongs to, and the pairs of a part in evaluation order: grouped
+// by primitive direction.
+template <int M>
+struct Part64 {
+  int n;                          // pairs
+  int dir[Model<M>::NP];          // direction of +e (e = k b; -e follows it)
+  int b[Model<M>::NP][3];
+  int k[Model<M>::NP];
+  int grp[Model<M>::NP];
+};
+
+// D2Q33 (4 pairs each): (1,0) (2,0) | (1,1) (3,0) | (2,2) (4,4) | (2,1).
+// D3Q95 (11 or 12 pairs): (2,2,0) (3,3,0) | (2,0,0) (3,0,0) (4,4,0) |
+//   (2,2,2) (3,3,3) (5,0,0) | (2,2,5).  Shell numbers as in velset.cuh.
+template <int M>
+LBM_HD constexpr int shell_part64(int g) {
+  constexpr int d2[8] = {-1, 0, 1, 0, 2, 1, 3, 2};
+  constexpr int d3[10] = {-1, 1, 0, 2, 1, 0, 2, 3, 1, 2};
+  return M == 0 ? d2[g] : d3[g];
+}
+
+template <int M>
+LBM_HD constexpr Part64<M> make_part64(int part) {
+  using Mo = Model<M>;
+  Part64<M> t{};
+  bool used[Mo::NP] = {};
+  for (int p0 = 0; p0 < Mo::NP; ++p0) {
+    if (used[p0] || shell_part64<M>(Mo::vs.grp[1 + 2 * p0]) != part) continue;
+    const int* e0 = Mo::vs.e[1 + 2 * p0];
+    const int g0 = igcd(igcd(iabs(e0[0]), iabs(e0[1])), iabs(e0[2]));
+    for (int p = p0; p < Mo::NP; ++p) {          // the part's pairs along e0
+      const int* e = Mo::vs.e[1 + 2 * p];
+      const int g = igcd(igcd(iabs(e[0]), iabs(e[1])), iabs(e[2]));
+      if (used[p] || shell_part64<M>(Mo::vs.grp[1 + 2 * p]) != part) continue;
+      if (e[0] * g0 != e0[0] * g || e[1] * g0 != e0[1] * g || e[2] * g0 != e0[2] * g) continue;
+      used[p] = true;
+      t.dir[t.n] = 1 + 2 * p;
+      for (int d = 0; d < 3; ++d) t.b[t.n][d] = e[d] / g;
+      t.k[t.n] = g;
+      t.grp[t.n] = Mo::vs.grp[1 + 2 * p];
+      ++t.n;
+    }
+  }
+  return t;
+}
+
+template <int M, int P>
+struct P64 {
+  static constexpr Part64<M> t = make_part64<M>(P);
+  static constexpr bool first_of(int n) {        // first / last pair of its shell
+    for (int m = 0; m < n; ++m)
+      if (t.grp[m] == t.grp[n]) return false;
+    return true;
+  }
+  static constexpr bool last_of(int n) {
+    for (int m = n + 1; m < t.n; ++m)
+      if (t.grp[m] == t.grp[n]) return false;
+    return true;
+  }
+  static constexpr bool new_base(int n) {
+    return n == 0 || t.b[n][0] != t.b[n - 1][0] || t.b[n][1] != t.b[n - 1][1] ||
+           t.b[n][2] != t.b[n - 1][2];
+  }
+};
+static_assert(P64<0, 0>::t.n == 4 && P64<0, 1>::t.n == 4 && P64<0, 2>::t.n == 4 &&
+              P64<0, 3>::t.n == 4, "D2Q33 parts");
+static_assert(P64<1, 0>::t.n == 12 && P64<1, 1>::t.n == 12 && P64<1, 2>::t.n == 11 &&
+              P64<1, 3>::t.n == 12, "D3Q95 parts");
+
+// sum w h, sum w h |xi|^2 and sum w h e over one part.
+struct Mom64 {
+  double r, e, x, y, z;
+};
+template <int M>
+__device__ __forceinline__ Mom64 add64(const Mom64& a, const Mom64& b) {
+  return {__dadd_rn(a.r, b.r), __dadd_rn(a.e, b.e), __dadd_rn(a.x, b.x), __dadd_rn(a.y, b.y),
+          Model<M>::D == 3 ? __dadd_rn(a.z, b.z) : 0.0};
+}
+
+template <int M, int P, class Get>
+__device__ __forceinline__ Mom64 moments64(Get&& hv) {
+  using T = P64<M, P>;
+  const ModelConst& mc = c_mc[M];
+  Mom64 m = {0.0, 0.0, 0.0, 0.0, 0.0};
+  bool none = true;
+  double gs[Model<M>::G], gx[Model<M>::G], gy[Model<M>::G], gz[Model<M>::G];
+  sfor<0, T::t.n>([&](auto I) {
+    constexpr int n = decltype(I)::value;
+    constexpr int g = T::t.grp[n], i = T::t.dir[n];
+    constexpr int bx = T::t.b[n][0], by = T::t.b[n][1], bz = T::t.b[n][2];
+    const double hp = hv(std::integral_constant<int, i>{});
+    const double hm = hv(std::integral_constant<int, i + 1>{});
+    const double sp = __dadd_rn(hp, hm), dm = __dsub_rn(hp, hm);
+    if constexpr (T::first_of(n)) {
+      gs[g] = sp;
+      gx[g] = gy[g] = gz[g] = 0.0;
+    } else {
+      gs[g] = __dadd_rn(gs[g], sp);
+    }
+    if constexpr (bx != 0) gx[g] = xaxpy<bx>(dm, gx[g]);
+    if constexpr (by != 0) gy[g] = xaxpy<by>(dm, gy[g]);
+    if constexpr (bz != 0) gz[g] = xaxpy<bz>(dm, gz[g]);
+    if constexpr (T::last_of(n)) {
+      m.r = none ? __dmul_rn(mc.W[g], gs[g]) : __fma_rn(mc.W[g], gs[g], m.r);
+      m.e = none ? __dmul_rn(mc.WX2[g], gs[g]) : __fma_rn(mc.WX2[g], gs[g], m.e);
+      m.x = none ? __dmul_rn(mc.Wk[g], gx[g]) : __fma_rn(mc.Wk[g], gx[g], m.x);
+      m.y = none ? __dmul_rn(mc.Wk[g], gy[g]) : __fma_rn(mc.Wk[g], gy[g], m.y);
+      if constexpr (Model<M>::D == 3)
+        m.z = none ? __dmul_rn(mc.Wk[g], gz[g]) : __fma_rn(mc.Wk[g], gz[g], m.z);
+      none = false;
+    }
+  });
+  return m;
+}
+
+// What the relaxation needs of a cell: the velocity a u (s = e . v), and the equilibrium's
+// coefficients with rho folded in.  h^eq of a pair +- k b, with s = b . v, is
+//   c0 +- s c1 + s^2 c2 +- s^3 c3 + s^4 c4
+//   c0 = P0 + x2 K1 + (x2^2 / 8) tt,  c1 = k L0 + (k x2 / 2) rt,
+//   c2 = (k^2 / 2) d + (k^2 x2 / 4) rt,  c3 = (k^3 / 6) rho,  c4 = (k^4 / 24) rho
+// (EqCoef's polynomials times rho; rt = rho t, tt = rho t^2, d = L0 - rt).
+struct Cell64 {
+  double vx, vy, vz;
+  double P0, K1, tt, L0, rt, d, rho;
+};
+template <int M>
+__device__ __forceinline__ Cell64 cell64(const Mom64& m) {
+  constexpr int D = Model<M>::D;
+  const double a = c_mc[M].a;
+  Cell64 c;
+  c.rho = __dadd_rn(1.0, m.r);
+  const double ir = 1.0 / c.rho;
+  const double air = __dmul_rn(a, ir);
+  const double ux = __dmul_rn(air, m.x), uy = __dmul_rn(air, m.y);
+  const double uz = D == 3 ? __dmul_rn(air, m.z) : 0.0;
+  double q = __fma_rn(ux, ux, __dmul_rn(uy, uy));
+  if constexpr (D == 3) q = __fma_rn(uz, uz, q);
+  // theta - 1 = ((E - D rho) / rho - |u|^2) / D
+  const double t = __dmul_rn(__fma_rn(__fma_rn(-(double)D, m.r, m.e), ir, -q), 1.0 / D);
+  c.vx = __dmul_rn(a, ux);
+  c.vy = __dmul_rn(a, uy);
+  c.vz = D == 3 ? __dmul_rn(a, uz) : 0.0;
+  c.rt = __dmul_rn(c.rho, t);
+  c.tt = __dmul_rn(c.rt, t);
+  const double K0m1 =
+      __fma_rn(t, __fma_rn(t, 0.125 * D * (D + 2), __fma_rn(q, 0.25 * (D + 2), -0.5 * D)),
+               __dmul_rn(q, __fma_rn(q, 0.125, -0.5)));
+  c.P0 = __fma_rn(c.rho, K0m1, m.r);
+  c.K1 = __dmul_rn(c.rt, __fma_rn(t, -0.25 * (D + 2), __fma_rn(q, -0.25, 0.5)));
+  c.L0 = __fma_rn(c.rt, -0.5 * (D + 2), __dmul_rn(c.rho, __fma_rn(q, -0.5, 1.0)));
+  c.d = __dsub_rn(c.L0, c.rt);
+  return c;
+}
+
+// The relaxation h' = h + omega (h^eq - h) of one part's pairs.
+template <int M, int P, class Get, class Store>
+__device__ __forceinline__ void relax64(const Cell64& c, double omega, Get&& hv, Store&& st) {
+  using T = P64<M, P>;
+  const ModelConst& mc = c_mc[M];
+  double s = 0.0, s2 = 0.0;
+  sfor<0, T::t.n>([&](auto I) {
+    constexpr int n = decltype(I)::value;
+    constexpr int g = T::t.grp[n], k = T::t.k[n], i = T::t.dir[n];
+    if constexpr (T::new_base(n)) {
+      s = edot<double, T::t.b[n][0], T::t.b[n][1], T::t.b[n][2]>(c.vx, c.vy, c.vz);
+      s2 = __dmul_rn(s, s);
+    }
+    // the shell's coefficients: the same expressions for each of its pairs, which the
+    // compiler forms once
+    const double c0 = __fma_rn(mc.X4o8[g], c.tt, __fma_rn(mc.X2[g], c.K1, c.P0));
+    const double c1 = __fma_rn(mc.kX2o2[g], c.rt, __dmul_rn((double)k, c.L0));
+    const double c2 = __fma_rn(mc.k2X2o4[g], c.rt, __dmul_rn(0.5 * k * k, c.d));
+    const double c3 = __dmul_rn(k * k * k / 6.0, c.rho);
+    const double c4 = __dmul_rn(k * k * k * k / 24.0, c.rho);
+    const double ev = __fma_rn(s2, __fma_rn(s2, c4, c2), c0);
+    const double od = __dmul_rn(s, __fma_rn(s2, c3, c1));
+    const double hp = hv(std::integral_constant<int, i>{});
+    const double hm = hv(std::integral_constant<int, i + 1>{});
+    st(std::integral_constant<int, i>{}, __fma_rn(omega, __dsub_rn(__dadd_rn(ev, od), hp), hp));
+    st(std::integral_constant<int, i + 1>{}, __fma_rn(omega, __dsub_rn(__dsub_rn(ev, od), hm), hm));
+  });
+}
+
+// The four parts' sums and the rest direction (deviation h0).
+template <int M>
+__device__ __forceinline__ Mom64 total64(const Mom64& p01, const Mom64& p23, double h0) {
+  Mom64 m = add64<M>(p01, p23);
+  m.r = __fma_rn(c_mc[M].W[0], h0, m.r);
+  return m;
+}
+__device__ __forceinline__ double relax_rest64(const Cell64& c, double omega, double h0) {
+  return __fma_rn(omega, __dsub_rn(c.P0, h0), h0);
+}
+
+// a3 - a6 of one cell by one thread: hm(I) / hr(I) return direction I's population for
+// the moments and for the relaxation (the same values; a kernel may read them again).
+template <int M, class GetM, class GetR, class Store>
+__device__ __forceinline__ void collide64(GetM&& hm, GetR&& hr, double omega, Store&& st) {
+  constexpr std::integral_constant<int, 0> rest{};
+  const Mom64 p0 = moments64<M, 0>(hm), p1 = moments64<M, 1>(hm);
+  const Mom64 p01 = add64<M>(p0, p1);
+  const Mom64 p2 = moments64<M, 2>(hm), p3 = moments64<M, 3>(hm);
+  const Cell64 c = cell64<M>(total64<M>(p01, add64<M>(p2, p3), hm(rest)));
+  st(rest, relax_rest64(c, omega, hr(rest)));
+  relax64<M, 0>(c, omega, hr, st);
+  relax64<M, 1>(c, omega, hr, st);
+  relax64<M, 2>(c, omega, hr, st);
+  relax64<M, 3>(c, omega, hr, st);
+}
+
+}  // namespace lbm

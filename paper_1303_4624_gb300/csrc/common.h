@@ -14,6 +14,10 @@ constexpr int kMaxGc = 10;
 struct ModelConst {
   double W[kMaxGc];    // weight of each symmetry group
   double X2[kMaxGc];   // |xi|^2 = a^2 |e|^2 of each group
+  double WX2[kMaxGc];  // W X2
+  // with k the gcd of the group's components (e = k b, b primitive):
+  double Wk[kMaxGc];   // W k
+  double X4o8[kMaxGc], kX2o2[kMaxGc], k2X2o4[kMaxGc];   // X2^2 / 8, k X2 / 2, k^2 X2 / 4
   float Wf[kMaxGc];
   float X2f[kMaxGc];
   float X2lo[kMaxGc];  // X2 - X2f: with X2f, X2 as a double-float (hi, lo) pair

@@ -2,6 +2,7 @@
 // k_fp32.cu, k_fp16.cu and k_bf16.cu after defining LBM_STORE (element type) and
 // LBM_OPS (name of the StorageOps table).
 #include <algorithm>
+#include <atomic>
 #include <mutex>
 
 #include "kernels.cuh"
@@ -166,6 +167,47 @@ DirectFn direct_kernel(const Grid& g, int rev) {
   return rev ? k_stream_collide<M, S, true, false> : k_stream_collide<M, S, false, false>;
 }
 
+// SMs of the current device (looked up once per device).
+cudaError_t sm_count(int* sms) {
+  static std::atomic<int> known[16];
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  int v = dev < 16 ? known[dev].load() : 0;
+  if (v == 0) {
+    e = cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 16) known[dev].store(v);
+  }
+  *sms = v;
+  return cudaSuccess;
+}
+
+// The FP64 kernel: 32 cells per block, 1, 2 or 4 warps (lin64_warps).
+template <int M>
+cudaError_t step64_m(const void* src, void* dst, const Grid& g, double omega, int rev,
+                     cudaStream_t st) {
+  int sms = 0;
+  cudaError_t e = sm_count(&sms);
+  if (e != cudaSuccess) return e;
+  const int w = lin64_warps<M>(g.ncell, sms);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)((g.ncell + 31) / 32));
+  cfg.blockDim = dim3(32 * w);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  auto kern = k_stream_collide64<M, false, 1>;
+  if (w == 1) kern = rev ? k_stream_collide64<M, true, 1> : k_stream_collide64<M, false, 1>;
+  else if (w == 2) kern = k_stream_collide64<M, false, 2>;
+  else kern = k_stream_collide64<M, false, 4>;
+  return cudaLaunchKernelEx(&cfg, kern, static_cast<const double*>(src), static_cast<double*>(dst),
+                            g, omega);
+}
+
 template <int M>
 cudaError_t step_m(const void* src, void* dst, const Grid& g, double omega, int variant, int* status,
                    const StepTest* test, cudaStream_t st) {
@@ -184,6 +226,9 @@ cudaError_t step_m(const void* src, void* dst, const Grid& g, double omega, int 
       return cudaGetLastError();
     }
   }
+  if constexpr (std::is_same<S, double>::value) {
+    return step64_m<M>(src, dst, g, omega, rev, st);
+  } else {
   const int bx = cell_block_x(g.nx);
   const dim3 grid((unsigned)((g.nx + bx - 1) / bx), (unsigned)g.ny, (unsigned)g.nz);
 #ifndef LBM_NO_PDL
@@ -204,6 +249,7 @@ cudaError_t step_m(const void* src, void* dst, const Grid& g, double omega, int 
                                                 omega);
   return cudaGetLastError();
 #endif
+  }
 }
 
 template <int M>

@@ -481,6 +481,10 @@ __device__ __forceinline__ void half_collide(const CellState<Rt>& c, double omeg
   });
 }
 
+}  // namespace lbm
+#include "collide64.cuh"
+namespace lbm {
+
 // Arithmetic options per storage form: FP32 / FP64 storage keep per-pair Kahan sums
 // and the exact-fixed-point relaxation; FP16 / BF16 storage use per-shell
 // compensation and the two-term relaxation (see half_moments / half_collide).
@@ -499,6 +503,10 @@ struct FormOpts {
 template <int M, class S, class Rt, class GetM, class GetR, class Store>
 __device__ __forceinline__ void cell_collide_with2(GetM&& hm, GetR&& hr, double omega,
                                                    Store&& st) {
+  if constexpr (std::is_same<Rt, double>::value) {
+    collide64<M>(hm, hr, omega, st);
+    return;
+  } else {
   using Mo = Model<M>;
   constexpr int NP = Mo::NP, NH = NP / 2;
   constexpr bool SH = FormOpts<S>::kShell, EX = FormOpts<S>::kExact;
@@ -509,6 +517,7 @@ __device__ __forceinline__ void cell_collide_with2(GetM&& hm, GetR&& hr, double 
   // a5, a6
   half_collide<M, Rt, 0, NH, true, EX>(c, omega, hr, st);
   half_collide<M, Rt, NH, NP, false, EX>(c, omega, hr, st);
+  }
 }
 template <int M, class S, class Rt, class Get, class Store>
 __device__ __forceinline__ void cell_collide_with(Get&& hv, double omega, Store&& st) {
@@ -668,6 +677,117 @@ __global__ void __launch_bounds__(128, DirectMinBlocks<M, S>::value)
           Codec<S>::st(dst + (size_t)decltype(I)::value * (size_t)g.ncell + self, v);
         });
   }
+}
+
+// FP64 form: linear cell index (rows of any length fill the warps), 32 cells per block,
+// WARPS warps per block.  The FP64 pipe bounds the form (see collide64.cuh): each of an
+// SM's four schedulers takes 64 cycles an FP64 instruction, so the grid's time is that of
+// the scheduler with the most warps.  Blocks of one warp spread them evenly (256 x 8
+// D2Q33: 64 warps on as many SMs, against 16 SMs with four each); where even so there are
+// fewer warps than schedulers, WARPS = 2 or 4 warps share 32 cells: each takes some of the
+// parts of collide64, and the parts' moments are exchanged through shared memory and
+// summed in collide64's order, so every WARPS gives the same bits (see lin64_warps for
+// the rule).
+// The populations are read twice, for the moments and for the relaxation (D3Q95: 95
+// doubles would take 190 registers); the second read comes from L1 / L2, and memory has
+// the time (1520 bytes a cell at under 1 TB/s).
+__device__ __forceinline__ double ld_again(const double* p) {
+  double v;   // volatile: not merged with the first read
+  asm volatile("ld.global.nc.f64 %0, [%1];" : "=d"(v) : "l"(p));
+  return v;
+}
+template <int M, bool REV, int WARPS>
+__global__ void __launch_bounds__(32 * WARPS, 8 / WARPS)
+    k_stream_collide64(const double* __restrict__ src, double* __restrict__ dst, Grid g,
+                       double omega) {
+  using Mo = Model<M>;
+  constexpr int D = Mo::D, RR = Mo::R;
+  constexpr std::integral_constant<int, 0> rest{};
+  wait_prior_grid();
+  allow_next_grid();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const unsigned b = REV ? gridDim.x - 1 - blockIdx.x : blockIdx.x;
+  const unsigned cell = b * 32 + lane;
+  const bool active = cell < (unsigned)g.ncell;
+  if (WARPS == 1 && !active) return;
+  const unsigned at0 = active ? cell : 0;
+  const unsigned row = at0 / (unsigned)g.nx;
+  const int x = (int)(at0 - row * (unsigned)g.nx);
+  const int z = D == 3 ? (int)(row / (unsigned)g.ny) : 0;
+  const int y = (int)row - z * g.ny;
+  int xo[2 * RR + 1], yo[2 * RR + 1], zo[2 * RR + 1];
+  neighbour_offsets<D, RR>(x, y, z, g.nx, g.ny, g.nz, g.nxy, xo, yo, zo);
+  auto at = [&](auto I) {
+    constexpr int i = decltype(I)::value;
+    constexpr int ex = Mo::vs.e[i][0], ey = Mo::vs.e[i][1], ez = Mo::vs.e[i][2];
+    return src + (size_t)i * (size_t)g.ncell + (zo[ez + RR] + yo[ey + RR] + xo[ex + RR]);
+  };
+  auto st = [&](auto I, double v) {
+    if (active) dst[(size_t)decltype(I)::value * (size_t)g.ncell + cell] = v;
+  };
+  auto hm = [&](auto I) { return __ldg(at(I)); };
+  auto hr = [&](auto I) { return ld_again(at(I)); };
+  if constexpr (WARPS == 1) {
+    collide64<M>(hm, hr, omega, st);
+  } else {
+    constexpr int PW = kParts64 / WARPS;         // parts per warp
+    __shared__ double xch[kParts64 / PW][5][32];
+    const double h0 = hm(rest);
+    Mom64 mine;
+    sfor<0, WARPS>([&](auto Wi) {
+      constexpr int w = decltype(Wi)::value;
+      if (warp == w) {
+        mine = moments64<M, w * PW>(hm);
+        if constexpr (PW == 2) mine = add64<M>(mine, moments64<M, w * PW + 1>(hm));
+      }
+    });
+    xch[warp][0][lane] = mine.r;
+    xch[warp][1][lane] = mine.e;
+    xch[warp][2][lane] = mine.x;
+    xch[warp][3][lane] = mine.y;
+    xch[warp][4][lane] = mine.z;
+    __syncthreads();
+    auto part = [&](int p) {
+      return Mom64{xch[p][0][lane], xch[p][1][lane], xch[p][2][lane], xch[p][3][lane], xch[p][4][lane]};
+    };
+    Mom64 p01, p23;
+    if constexpr (PW == 2) {
+      p01 = part(0);
+      p23 = part(1);
+    } else {
+      p01 = add64<M>(part(0), part(1));
+      p23 = add64<M>(part(2), part(3));
+    }
+    const Cell64 c = cell64<M>(total64<M>(p01, p23, h0));
+    sfor<0, WARPS>([&](auto Wi) {
+      constexpr int w = decltype(Wi)::value;
+      if (warp == w) {
+        if constexpr (w == 0) st(rest, relax_rest64(c, omega, hr(rest)));
+        relax64<M, w * PW>(c, omega, hr, st);
+        if constexpr (PW == 2) relax64<M, w * PW + 1>(c, omega, hr, st);
+      }
+    });
+  }
+}
+
+// Warps per 32 cells: the choice with the fewest FP64 instructions on the busiest
+// scheduler, ceil(warps / schedulers) times the instructions of a warp.  Those are about
+// 200 / 830 for all pairs of D2Q33 / D3Q95 and 70 for what every warp repeats (moment
+// totals, 1 / rho, the coefficients of the cell).
+template <int M>
+inline int lin64_warps(long long ncell, int sms) {
+  const long long groups = (ncell + 31) / 32;
+  int best = 1;
+  long long best_cost = -1;
+  for (int w = 1; w <= 4; w *= 2) {
+    const long long rounds = (groups * w + 4LL * sms - 1) / (4LL * sms);
+    const long long cost = rounds * ((M == 0 ? 200 : 830) / w + 70);
+    if (best_cost < 0 || cost < best_cost) {
+      best = w;
+      best_cost = cost;
+    }
+  }
+  return best;
 }
 
 // ----------------------------------------------------------------- split kernel

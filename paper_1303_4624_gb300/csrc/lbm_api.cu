@@ -200,11 +200,17 @@ bool build_host_model(int model, HostModel* hm) {
   for (int g = 0; g < G; ++g) {
     mc.W[g] = hm->W[g];
     mc.X2[g] = a * a * vs.e2[g];
+    mc.WX2[g] = mc.W[g] * mc.X2[g];
     mc.Wf[g] = (float)mc.W[g];
     mc.X2f[g] = (float)mc.X2[g];
     mc.X2lo[g] = (float)(mc.X2[g] - (double)mc.X2f[g]);
   }
   for (int i = 0; i < vs.Q; ++i) {
+    const int g = vs.grp[i], k = igcd(igcd(iabs(vs.e[i][0]), iabs(vs.e[i][1])), iabs(vs.e[i][2]));
+    mc.Wk[g] = k * mc.W[g];
+    mc.X4o8[g] = mc.X2[g] * mc.X2[g] / 8.0;
+    mc.kX2o2[g] = k * mc.X2[g] / 2.0;
+    mc.k2X2o4[g] = k * k * mc.X2[g] / 4.0;
     mc.w[i] = hm->w[i];
     for (int d = 0; d < 3; ++d) {
       mc.e[i][d] = vs.e[i][d];

@@ -32,6 +32,14 @@ constexpr int kRepsD3Q95[10][3] = {{0, 0, 0}, {2, 0, 0}, {2, 2, 0}, {2, 2, 2}, {
                                    {3, 3, 0}, {3, 3, 3}, {2, 2, 5}, {4, 4, 0}, {5, 0, 0}};
 
 LBM_HD constexpr int iabs(int v) { return v < 0 ? -v : v; }
+LBM_HD constexpr int igcd(int a, int b) {
+  while (b) {
+    const int t = a % b;
+    a = b;
+    b = t;
+  }
+  return a;
+}
 
 template <int G>
 LBM_HD constexpr VelSet expand(const int (&reps)[G][3], int D) {
