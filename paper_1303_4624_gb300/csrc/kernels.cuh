@@ -1164,6 +1164,103 @@ __device__ __forceinline__ void moments_fp32_forms(const S* __restrict__ src, co
   }
 }
 
+// An order-preserving 64-bit key of a double: a < b exactly when key(a) < key(b).
+__device__ __forceinline__ long long order_key(double v) {
+  const long long b = __double_as_longlong(v);
+  return b ^ ((b >> 63) & 0x7fffffffffffffffll);
+}
+__device__ __forceinline__ double order_value(long long k) {
+  return __longlong_as_double(k ^ ((k >> 63) & 0x7fffffffffffffffll));
+}
+
+// Moments of the FP64 form, one thread per cell: collide64's sums (about 250 FP64
+// operations a D3Q95 cell; population by population, f = w (1 + h) and six sums each took
+// ~900, and bound the kernel at 317 us for 131,072 cells).  The minimum and the count of
+// non-finite populations are taken on the integer pipe (an FP64 minimum costs more than
+// three FP64 instructions), and each warp reduces one audit slot over the block.
+template <int M>
+__device__ __forceinline__ void moments_fp64_form(const double* __restrict__ src, const Grid& g,
+                                                  long long idx, long long end, long long block,
+                                                  double* __restrict__ rho_out,
+                                                  double* __restrict__ U_out,
+                                                  double* __restrict__ T_out,
+                                                  double* __restrict__ partials) {
+  constexpr int D = Model<M>::D;
+  const ModelConst& mc = c_mc[M];
+  const long long none = order_key(1e300);
+  long long hmin = none;
+  int bad = 0;
+  double rho = 0.0, e = 0.0;
+  Mom64 m = {};
+  const bool active = idx < end;
+  if (active) {
+    auto hv = [&](auto I) {
+      const double v = __ldg(src + (size_t)decltype(I)::value * (size_t)g.ncell + idx);
+      const int top = __double2hiint(v) & 0x7fffffff;
+      bad += top >= 0x7ff00000;                              // Inf or NaN
+      const bool nan = top > 0x7ff00000 || (top == 0x7ff00000 && __double2loint(v) != 0);
+      const long long k = order_key(v);
+      if (!nan && k < hmin) hmin = k;
+      return v;
+    };
+    const double h0 = hv(std::integral_constant<int, 0>{});
+    const Mom64 p0 = moments64<M, 0>(hv), p1 = moments64<M, 1>(hv);
+    const Mom64 p01 = add64<M>(p0, p1);
+    const Mom64 p2 = moments64<M, 2>(hv), p3 = moments64<M, 3>(hv);
+    m = total64<M>(p01, add64<M>(p2, p3), h0);
+    rho = 1.0 + m.r;
+    const double ir = 1.0 / rho;
+    auto over_rho = [&](double v) {                          // v / rho, one residual step
+      const double y = __dmul_rn(v, ir);
+      return __fma_rn(__fma_rn(-y, rho, v), ir, y);
+    };
+    const double Ux = over_rho(m.x), Uy = over_rho(m.y), Uz = D == 3 ? over_rho(m.z) : 0.0;
+    double U2 = __fma_rn(Ux, Ux, __dmul_rn(Uy, Uy));
+    if constexpr (D == 3) U2 = __fma_rn(Uz, Uz, U2);
+    // T = T0 + ((E - D rho) T0 / rho - |U|^2) / D
+    const double t = __dmul_rn(
+        __fma_rn(mc.T0, over_rho(__fma_rn(-(double)D, m.r, m.e)), -U2), 1.0 / D);
+    if (rho_out) rho_out[idx] = rho;
+    if (U_out) {
+      U_out[idx] = Ux;
+      U_out[g.ncell + idx] = Uy;
+      if (D == 3) U_out[2 * g.ncell + idx] = Uz;
+    }
+    if (T_out) T_out[idx] = __dadd_rn(mc.T0, t);
+    e = __dmul_rn(0.5 * mc.T0, __dadd_rn((double)D, m.e));
+  }
+  static_assert(kMomentThreads / 32 == kAuditSlots, "one warp per audit slot");
+  __shared__ double shv[kAuditSlots][kMomentThreads];
+  const int tid = threadIdx.x, lane = tid & 31, slot = tid >> 5;
+  shv[0][tid] = rho;
+  shv[1][tid] = m.x;
+  shv[2][tid] = m.y;
+  shv[3][tid] = m.z;
+  shv[4][tid] = e;
+  shv[5][tid] = __longlong_as_double(hmin);
+  shv[6][tid] = __longlong_as_double((long long)bad);
+  shv[7][tid] = __longlong_as_double((long long)active);
+  __syncthreads();
+  double out;
+  if (slot >= 5) {                                           // minimum and counts: integers
+    long long v = __double_as_longlong(shv[slot][lane]);
+    for (int c = lane + 32; c < kMomentThreads; c += 32) {
+      const long long w = __double_as_longlong(shv[slot][c]);
+      v = slot == 5 ? min(v, w) : v + w;
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+      const long long w = __shfl_xor_sync(0xffffffffu, v, o);
+      v = slot == 5 ? min(v, w) : v + w;
+    }
+    out = slot == 5 ? (v == none ? 1e300 : 1.0 + order_value(v)) : (double)v;
+  } else {
+    out = shv[slot][lane];
+    for (int c = lane + 32; c < kMomentThreads; c += 32) out += shv[slot][c];
+    out = warp_sum(out);
+  }
+  if (lane == 0) partials[(size_t)block * kAuditSlots + slot] = out;
+}
+
 template <class S>
 struct MomMinBlocks {
   static constexpr int value = std::is_same<S, double>::value ? 1 : LBM_MOM_MINB;
@@ -1176,56 +1273,12 @@ __global__ void __launch_bounds__(kMomentThreads, MomMinBlocks<S>::value)
     k_moments(const S* __restrict__ src, Grid g, double* __restrict__ rho_out,
               double* __restrict__ U_out, double* __restrict__ T_out,
               double* __restrict__ partials, long long block0, long long end) {
-  using Mo = Model<M>;
-  constexpr int D = Mo::D, Q = Mo::Q;
-  const ModelConst& mc = c_mc[M];
   const long long block = block0 + blockIdx.x;
   const long long idx = block * blockDim.x + threadIdx.x;
-  double acc[kAuditSlots] = {0, 0, 0, 0, 0, 1e300, 0, 0};
-  if constexpr (!std::is_same<S, double>::value) {
+  if constexpr (!std::is_same<S, double>::value)
     moments_fp32_forms<M, S>(src, g, idx, end, block, rho_out, U_out, T_out, partials);
-    return;
-  } else if (idx < end) {
-    double r = 0, mx = 0, my = 0, mz = 0, e2 = 0, mn = 1e300, bad = 0;
-    sfor<0, Q>([&](auto I) {
-      constexpr int i = decltype(I)::value;
-      constexpr int ex = Mo::vs.e[i][0], ey = Mo::vs.e[i][1], ez = Mo::vs.e[i][2];
-      const double hv = to_double(src[(size_t)i * g.ncell + idx]);
-      const double f = mc.w[i] * (1.0 + hv);
-      if (!isfinite(hv)) bad += 1.0;
-      mn = fmin(mn, 1.0 + hv);
-      r += f;
-      mx += ex * f;
-      my += ey * f;
-      mz += ez * f;
-      e2 += (ex * ex + ey * ey + ez * ez) * f;
-    });
-    const double Ux = mx / r, Uy = my / r, Uz = mz / r;
-    const double Tl = (e2 / r - (Ux * Ux + Uy * Uy + Uz * Uz)) / D;
-    if (rho_out) rho_out[idx] = r;
-    if (U_out) {
-      U_out[idx] = Ux;
-      U_out[g.ncell + idx] = Uy;
-      if (D == 3) U_out[2 * g.ncell + idx] = Uz;
-    }
-    if (T_out) T_out[idx] = Tl;
-    acc[0] = r; acc[1] = mx; acc[2] = my; acc[3] = mz; acc[4] = 0.5 * e2;
-    acc[5] = mn; acc[6] = bad; acc[7] = 1.0;
-  }
-  __shared__ double sh[kMomentThreads / 32][kAuditSlots];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-  for (int k = 0; k < kAuditSlots; ++k) {
-    const double v = (k == 5) ? warp_min(acc[k]) : warp_sum(acc[k]);
-    if (lane == 0) sh[wid][k] = v;
-  }
-  __syncthreads();
-  if (threadIdx.x < kAuditSlots) {
-    const int k = threadIdx.x;
-    double v = sh[0][k];
-    for (int w = 1; w < kMomentThreads / 32; ++w) v = (k == 5) ? fmin(v, sh[w][k]) : v + sh[w][k];
-    partials[(size_t)block * kAuditSlots + k] = v;
-  }
+  else
+    moments_fp64_form<M>(src, g, idx, end, block, rho_out, U_out, T_out, partials);
 }
 
 // Fixed-order reduction of the audit partials by one block of 256 threads.
