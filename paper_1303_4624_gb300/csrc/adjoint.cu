@@ -279,7 +279,7 @@ int lbm_backward(lbm_ctx* ctx, const double* dL_drhoN, double* dL_drho0, double*
     for (int64_t j = 0; j < k - 1; ++j)
       if ((rc = r.seg[j]->ensure(sb, v.stream))) return rc;
   }
-  const long long nblk = cell_blocks(v.g);
+  const long long nblk = v.ops->adjoint_blocks(v.g);
   if ((rc = r.nu[0].ensure(nb, v.stream)) || (rc = r.nu[1].ensure(nb, v.stream)) ||
       (rc = r.dldrho.ensure(n * sizeof(double), v.stream)) ||
       (rc = r.omega_acc.ensure((size_t)nblk * sizeof(double), v.stream)) ||

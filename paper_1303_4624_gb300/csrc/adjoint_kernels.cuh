@@ -5,6 +5,7 @@
 #pragma once
 
 #include "kernels.cuh"
+#include "contract.cuh"
 
 namespace lbm {
 
@@ -380,66 +381,242 @@ __global__ void __launch_bounds__(kAdjThreads, AdjMinBlocks<S>::value)
 
 #undef LBM_POP
 
-// dL/d(rho0, U0, T0): lambda_0(x, i) = nu0(x + e_i, i) contracted with the
-// derivatives of f_i^eq(rho, u, theta) at the initial fields (FP64).
+// The adjoint step of the FP64 form: the same derivatives as k_adjoint with the FP64
+// instructions counted (see collide64.cuh and contract.cuh): the forward moments shell by
+// shell, the contractions once per primitive vector; ~600 FP64 operations a D2Q33 cell
+// against ~900 pair by pair.  Linear cell index, 32 cells per block, shared by WARPS = 1, 2
+// or 4 warps as in k_stream_collide64.  State and lambda are read again where they are used
+// again; the FP64 pipe bounds the kernel and memory has the time.
+template <int M, bool kFirst, int WARPS>
+__global__ void __launch_bounds__(32 * WARPS, 8 / WARPS)
+    k_adjoint64(const double* __restrict__ state, const double* __restrict__ nu_next,
+                const double* __restrict__ dldrho, double* __restrict__ nu_out,
+                double* __restrict__ omega_acc, Grid g, double omega) {
+  using Mo = Model<M>;
+  constexpr int D = Mo::D, RR = Mo::R, PW = kParts64 / WARPS;
+  const ModelConst& mc = c_mc[M];
+  wait_prior_grid();
+  allow_next_grid();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const unsigned cell = blockIdx.x * 32u + lane;
+  const bool active = cell < (unsigned)g.ncell;
+  const unsigned at0 = active ? cell : 0;
+  const unsigned row = at0 / (unsigned)g.nx;
+  const int x = (int)(at0 - row * (unsigned)g.nx);
+  const int z = D == 3 ? (int)(row / (unsigned)g.ny) : 0;
+  const int y = (int)row - z * g.ny;
+  int xo[2 * RR + 1], yo[2 * RR + 1], zo[2 * RR + 1];
+  neighbour_offsets<D, RR>(x, y, z, g.nx, g.ny, g.nz, g.nxy, xo, yo, zo);
+  const size_t nc = (size_t)g.ncell;
+  auto hv = [&](auto I) {                  // gathered from x - e_i
+    constexpr int i = decltype(I)::value;
+    constexpr int ex = Mo::vs.e[i][0], ey = Mo::vs.e[i][1], ez = Mo::vs.e[i][2];
+    return __ldg(state + (size_t)i * nc + (zo[ez + RR] + yo[ey + RR] + xo[ex + RR]));
+  };
+  const double l1 = kFirst ? dldrho[at0] : 0.0;
+  auto lam = [&](auto I) -> double {       // nu_next(x + e_i, i)
+    constexpr int i = decltype(I)::value;
+    constexpr int ex = Mo::vs.e[i][0], ey = Mo::vs.e[i][1], ez = Mo::vs.e[i][2];
+    if constexpr (kFirst) return l1;
+    else return ld_again(nu_next + (size_t)i * nc + (zo[RR - ez] + yo[RR - ey] + xo[RR - ex]));
+  };
+  __shared__ double xch[WARPS][7][32];
+  // sums over the warps, in order; the value of warp w is in xch[w][k]
+  auto total = [&](int k) {
+    double v = xch[0][k][lane];
+    for (int w = 1; w < WARPS; ++w) v = __dadd_rn(v, xch[w][k][lane]);
+    return v;
+  };
+
+  // pass 1: forward moments, and sum w lambda h over the pairs
+  Mom64 m = {};
+  double lh = 0.0;
+  auto dot = [&](auto Pi) {
+    using T = P64<M, decltype(Pi)::value>;
+    double gl[Mo::G];
+    sfor<0, T::t.n>([&](auto I) {
+      constexpr int n = decltype(I)::value, gg = T::t.grp[n], i = T::t.dir[n];
+      constexpr std::integral_constant<int, i> ip{};
+      constexpr std::integral_constant<int, i + 1> im{};
+      const double p = T::first_of(n) ? __dmul_rn(lam(ip), hv(ip)) : __fma_rn(lam(ip), hv(ip), gl[gg]);
+      gl[gg] = __fma_rn(lam(im), hv(im), p);
+      if constexpr (T::last_of(n)) lh = __fma_rn(mc.W[gg], gl[gg], lh);
+    });
+  };
+  auto pass1 = [&](auto Wi) {
+    constexpr int p0 = decltype(Wi)::value * PW;
+    m = moments64<M, p0>(hv);
+    dot(std::integral_constant<int, p0>{});
+    sfor<1, PW>([&](auto K) {
+      constexpr int p = p0 + decltype(K)::value;
+      m = add64<M>(m, moments64<M, p>(hv));
+      dot(std::integral_constant<int, p>{});
+    });
+  };
+  sfor<0, WARPS>([&](auto Wi) {
+    if (warp == decltype(Wi)::value) pass1(Wi);
+  });
+  if constexpr (WARPS > 1) {
+    xch[warp][0][lane] = m.r;
+    xch[warp][1][lane] = m.e;
+    xch[warp][2][lane] = m.x;
+    xch[warp][3][lane] = m.y;
+    xch[warp][4][lane] = m.z;
+    xch[warp][5][lane] = lh;
+    __syncthreads();
+    m = {total(0), total(1), total(2), total(3), D == 3 ? total(4) : 0.0};
+    lh = total(5);
+    __syncthreads();
+  }
+  const double h0 = hv(std::integral_constant<int, 0>{}), lam0 = lam(std::integral_constant<int, 0>{});
+  m.r = __fma_rn(mc.W[0], h0, m.r);
+  const double rho = 1.0 + m.r, ir = 1.0 / rho, a = mc.a;
+  const double ux = a * m.x * ir, uy = a * m.y * ir, uz = D == 3 ? a * m.z * ir : 0.0;
+  const double q = ux * ux + uy * uy + uz * uz;
+  const double t = ((m.e - D * m.r) * ir - q) * (1.0 / D);
+  // EqCoef's L0, L1, M0, M1
+  const double L1 = 0.5 * t, M1 = 0.25 * t;
+  const double L0 = fma(t, -0.5 * (D + 2), fma(q, -0.5, 1.0));
+  const double M0 = fma(t, -0.5, 0.5 * L0);
+
+  // pass 2: contractions of lambda
+  const ContractCell<double> cc = {a * ux, a * uy, a * uz, L0, L1, 2.0 * M0, L1, a * a};
+  double s6[7] = {};                       // Lr, Sq, St, V, sum w lambda
+  auto pass2 = [&](auto Pi) {
+    constexpr int p = decltype(Pi)::value;
+    Contraction<double> o = contract<M, P64<M, p>, double>(cc, lam);
+    if constexpr (p == 0) o.a0 = __fma_rn(mc.W[0], lam0, o.a0);
+    return o;
+  };
+  auto sum2 = [&](auto Wi) {
+    constexpr int p0 = decltype(Wi)::value * PW;
+    Contraction<double> o = pass2(std::integral_constant<int, p0>{});
+    sfor<1, PW>([&](auto K) {
+      const Contraction<double> w = pass2(std::integral_constant<int, p0 + decltype(K)::value>{});
+      o = {o.a0 + w.a0, o.x2 + w.x2, o.x4 + w.x4, o.S1c + w.S1c, o.S1e + w.S1e, o.S2b + w.S2b,
+           o.S2d + w.S2d, o.S3 + w.S3, o.S4 + w.S4, o.Vx + w.Vx, o.Vy + w.Vy, o.Vz + w.Vz};
+    });
+    contract_finish<D, double>(o, q, t, L0, L1, M0, M1, s6[0], s6[1], s6[2]);
+    s6[3] = o.Vx;
+    s6[4] = o.Vy;
+    s6[5] = o.Vz;
+    s6[6] = o.a0;
+  };
+  sfor<0, WARPS>([&](auto Wi) {
+    if (warp == decltype(Wi)::value) sum2(Wi);
+  });
+  if constexpr (WARPS > 1) {
+#pragma unroll
+    for (int k = 0; k < 7; ++k) xch[warp][k][lane] = s6[k];
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 7; ++k) s6[k] = total(k);
+  }
+  const double Lr = s6[0], Sq = s6[1], St = s6[2], Vx = s6[3], Vy = s6[4], Vz = s6[5];
+  // chain rule to the moments (as in k_adjoint)
+  const double Lux = rho * (a * Vx + 2.0 * ux * Sq), Luy = rho * (a * Vy + 2.0 * uy * Sq);
+  const double Luz = D == 3 ? rho * (a * Vz + 2.0 * uz * Sq) : 0.0;
+  const double Lt = rho * St, iDr = ir * (1.0 / D);
+  const double alpha = Lr - (ux * Lux + uy * Luy + uz * Luz) * ir + Lt * (q - D * (1.0 + t)) * iDr;
+  const double bx = Lux * ir - 2.0 * Lt * ux * iDr, by = Luy * ir - 2.0 * Lt * uy * iDr;
+  const double bz = Luz * ir - 2.0 * Lt * uz * iDr;
+  const double gam = Lt * iDr;
+
+  // pass 3: nu_n(x, j)
+  const double om1 = 1.0 - omega;
+  const double oa = omega * alpha, og = omega * gam, oma = omega * a;
+  const double obx = oma * bx, oby = oma * by, obz = oma * bz;
+  auto pass3 = [&](auto Pi) {
+    using T = P64<M, decltype(Pi)::value>;
+    double od = 0.0;
+    sfor<0, T::t.n>([&](auto I) {
+      constexpr int n = decltype(I)::value, i = T::t.dir[n], gg = T::t.grp[n], k = T::t.k[n];
+      if constexpr (T::new_base(n))
+        od = edot<double, T::t.b[n][0], T::t.b[n][1], T::t.b[n][2]>(obx, oby, obz);
+      const double ev = __fma_rn(og, mc.X2[gg], oa);
+      const double vp = __fma_rn((double)k, od, ev), vm = __fma_rn(-(double)k, od, ev);
+      const double lp = lam(std::integral_constant<int, i>{});
+      const double lm = lam(std::integral_constant<int, i + 1>{});
+      if (active) {
+        nu_out[(size_t)i * nc + cell] = __fma_rn(om1, lp, vp);
+        nu_out[(size_t)(i + 1) * nc + cell] = __fma_rn(om1, lm, vm);
+      }
+    });
+  };
+  sfor<0, WARPS>([&](auto Wi) {
+    constexpr int w = decltype(Wi)::value;
+    if (warp == w) sfor<0, PW>([&](auto K) { pass3(std::integral_constant<int, w * PW + decltype(K)::value>{}); });
+  });
+  if (warp == 0) {
+    if (active) nu_out[cell] = __fma_rn(om1, lam0, oa);
+    // dL/domega: rho Lr - sum w lambda (1 + h)
+    const double om = rho * Lr - (s6[6] + __fma_rn(mc.W[0] * lam0, h0, lh));
+    const double sum = warp_sum(active ? om : 0.0);
+    if (lane == 0) omega_acc[blockIdx.x] += sum;
+  }
+}
+
+// dL/d(rho0, U0, T0): lambda_0(x, i) = nu0(x + e_i, i) contracted with the derivatives of
+// f_i^eq(rho, u, theta) at the initial fields: FP64 for the FP64 form; double-float on the
+// FP32 pipe for the others, whose lambda is FP32 (~48 significant bits, against lambda's
+// 24).  In FP64 the contraction is bound by the FP64 pipe (64 cycles an instruction and
+// scheduler): 9.8 ms for 128^3 D3Q95 cells, as long as 22 adjoint steps.
 template <int M, class L>
 __global__ void __launch_bounds__(128)
     k_grad_init(const L* __restrict__ nu0, const double* __restrict__ fields,
                 double* __restrict__ d_rho, double* __restrict__ d_U, double* __restrict__ d_T,
                 Grid g) {
   using Mo = Model<M>;
-  constexpr int D = Mo::D, RR = Mo::R, NP = Mo::NP;
+  constexpr int D = Mo::D, RR = Mo::R;
+  constexpr bool kFF = std::is_same<L, float>::value;
+  using R = typename std::conditional<kFF, FF, double>::type;
   const ModelConst& mc = c_mc[M];
-  const int x = blockIdx.x * blockDim.x + threadIdx.x;
-  if (x >= g.nx) return;
-  const int y = blockIdx.y, z = blockIdx.z;
+  const unsigned cell = blockIdx.x * blockDim.x + threadIdx.x;
+  if (cell >= (unsigned)g.ncell) return;
+  const unsigned row = cell / (unsigned)g.nx;
+  const int x = (int)(cell - row * (unsigned)g.nx);
+  const int z = D == 3 ? (int)(row / (unsigned)g.ny) : 0;
+  const int y = (int)row - z * g.ny;
   int xo[2 * RR + 1], yo[2 * RR + 1], zo[2 * RR + 1];
   neighbour_offsets<D, RR>(x, y, z, g.nx, g.ny, g.nz, g.nxy, xo, yo, zo);
-  const size_t self = ((size_t)z * g.ny + y) * g.nx + x;
   const size_t n = (size_t)g.ncell;
-  const double rho = fields[self];
-  const double ux = mc.a * fields[n + self], uy = mc.a * fields[2 * n + self];
-  const double uz = (D == 3) ? mc.a * fields[3 * n + self] : 0.0;
-  const double theta = fields[(size_t)(D + 1) * n + self] / mc.T0;
-  const double q = ux * ux + uy * uy + uz * uz, t = theta - 1.0;
-  const EqCoef<double, D> cf(q, t);
-  const EqGrad<double, D> gr(q, t);
-  const double uax = mc.a * ux, uay = mc.a * uy, uaz = mc.a * uz;
-  const double l0 = (double)nu0[self];
-  double Lr = mc.W[0] * l0 * cf.K0, Sq = mc.W[0] * l0 * gr.Bq(0.0), St = mc.W[0] * l0 * gr.Bt(0.0);
-  double Vx = 0, Vy = 0, Vz = 0;
-  sfor<0, NP>([&](auto P) {
-    constexpr int p = decltype(P)::value;
-    constexpr int ip = 1 + 2 * p, im = 2 + 2 * p;
-    constexpr int gg = Mo::vs.grp[ip];
-    constexpr int ex = Mo::vs.e[ip][0], ey = Mo::vs.e[ip][1], ez = Mo::vs.e[ip][2];
-    const int cm = zo[ez + RR] + yo[ey + RR] + xo[ex + RR];
-    const int cp = zo[RR - ez] + yo[RR - ey] + xo[RR - ex];
-    const double lp = (double)nu0[(size_t)ip * n + cp];
-    const double lm = (double)nu0[(size_t)im * n + cm];
-    const double x2 = mc.X2[gg], w = mc.W[gg];
-    const double s = ex * uax + ey * uay + ez * uaz, s2 = s * s;
-    const double A1 = cf.A1(x2), A2 = cf.A2(x2);
-    const double Pe = cf.A0(x2) + s2 * (A2 + s2 / 24.0), Po = s * (A1 + s2 / 6.0);
-    const double Pse = A1 + 0.5 * s2, Pso = s * (2.0 * A2 + s2 / 6.0);
-    const double Pqe = gr.Bq(x2) - 0.25 * s2, Pqo = -0.5 * s;
-    const double Pte = gr.Bt(x2) + EqGrad<double, D>::Dt(x2) * s2, Pto = EqGrad<double, D>::Ct(x2) * s;
-    const double ls = lp + lm, ld = lp - lm;
-    Lr += w * (ls * Pe + ld * Po);
-    Sq += w * (ls * Pqe + ld * Pqo);
-    St += w * (ls * Pte + ld * Pto);
-    const double v = w * (ld * Pse + ls * Pso);
-    Vx += ex * v;
-    Vy += ey * v;
-    Vz += ez * v;
-  });
-  if (d_rho) d_rho[self] = Lr;
+  auto field = [&](int k) -> R {
+    if constexpr (kFF) return ff_from(fields[k * n + cell]); else return fields[k * n + cell];
+  };
+  R a, iT0;
+  if constexpr (kFF) { a = {mc.af, mc.alo}; iT0 = {mc.iT0f, mc.iT0lo}; }
+  else { a = mc.a; iT0 = 1.0 / mc.T0; }
+  const R rho = field(0);
+  const R ux = nmul(a, field(1)), uy = nmul(a, field(2));
+  const R uz = D == 3 ? nmul(a, field(3)) : ncst<R>(0.0);
+  const R t = nadd(nmul(iT0, field(D + 1)), ncst<R>(-1.0));
+  R q = nfma(ux, ux, nmul(uy, uy));
+  if constexpr (D == 3) q = nfma(uz, uz, q);
+  const R L1 = nmul(ncst<R>(0.5), t), M1 = nmul(ncst<R>(0.25), t);
+  const R L0 = nsub(nsub(ncst<R>(1.0), nmul(ncst<R>(0.5), q)), nmul(ncst<R>(0.5 * (D + 2)), t));
+  const R M0 = nmul(ncst<R>(0.5), nsub(L0, t));
+  const ContractCell<R> cc = {nmul(a, ux), nmul(a, uy), nmul(a, uz), L0, L1, nsub(L0, t), L1, nmul(a, a)};
+  auto lam = [&](auto I) -> R {
+    constexpr int i = decltype(I)::value;
+    constexpr int ex = Mo::vs.e[i][0], ey = Mo::vs.e[i][1], ez = Mo::vs.e[i][2];
+    const L v = __ldg(nu0 + (size_t)i * n + (zo[RR - ez] + yo[RR - ey] + xo[RR - ex]));
+    if constexpr (kFF) return FF{v, 0.f}; else return v;
+  };
+  Contraction<R> o = contract<M, P64<M, -1>, R>(cc, lam);
+  o.a0 = nfma(ShellW<R>::W(mc, 0), lam(std::integral_constant<int, 0>{}), o.a0);
+  R Lr, Sq, St;
+  contract_finish<D, R>(o, q, t, L0, L1, M0, M1, Lr, Sq, St);
+  auto put = [&](double* p, size_t at, R v) {
+    if constexpr (kFF) p[at] = ff_to_double(v); else p[at] = v;
+  };
+  if (d_rho) put(d_rho, cell, Lr);
   if (d_U) {
-    d_U[self] = mc.a * rho * (mc.a * Vx + 2.0 * ux * Sq);
-    d_U[n + self] = mc.a * rho * (mc.a * Vy + 2.0 * uy * Sq);
-    if (D == 3) d_U[2 * n + self] = mc.a * rho * (mc.a * Vz + 2.0 * uz * Sq);
+    const R ar = nmul(a, rho), Sq2 = nmul(ncst<R>(2.0), Sq);
+    put(d_U, cell, nmul(ar, nfma(a, o.Vx, nmul(ux, Sq2))));
+    put(d_U, n + cell, nmul(ar, nfma(a, o.Vy, nmul(uy, Sq2))));
+    if constexpr (D == 3) put(d_U, 2 * n + cell, nmul(ar, nfma(a, o.Vz, nmul(uz, Sq2))));
   }
-  if (d_T) d_T[self] = rho * St / mc.T0;
+  if (d_T) put(d_T, cell, nmul(nmul(rho, St), iT0));
 }
 
 // Fixed-order sum of n FP64 partials by one block of 256 threads.

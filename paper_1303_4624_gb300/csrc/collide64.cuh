@@ -47,19 +47,20 @@ LBM_HD constexpr int shell_part64(int g) {
   return M == 0 ? d2[g] : d3[g];
 }
 
+// part < 0: all pairs.
 template <int M>
 LBM_HD constexpr Part64<M> make_part64(int part) {
   using Mo = Model<M>;
   Part64<M> t{};
   bool used[Mo::NP] = {};
   for (int p0 = 0; p0 < Mo::NP; ++p0) {
-    if (used[p0] || shell_part64<M>(Mo::vs.grp[1 + 2 * p0]) != part) continue;
+    if (used[p0] || (part >= 0 && shell_part64<M>(Mo::vs.grp[1 + 2 * p0]) != part)) continue;
     const int* e0 = Mo::vs.e[1 + 2 * p0];
     const int g0 = igcd(igcd(iabs(e0[0]), iabs(e0[1])), iabs(e0[2]));
     for (int p = p0; p < Mo::NP; ++p) {          // the part's pairs along e0
       const int* e = Mo::vs.e[1 + 2 * p];
       const int g = igcd(igcd(iabs(e[0]), iabs(e[1])), iabs(e[2]));
-      if (used[p] || shell_part64<M>(Mo::vs.grp[1 + 2 * p]) != part) continue;
+      if (used[p] || (part >= 0 && shell_part64<M>(Mo::vs.grp[1 + 2 * p]) != part)) continue;
       if (e[0] * g0 != e0[0] * g || e[1] * g0 != e0[1] * g || e[2] * g0 != e0[2] * g) continue;
       used[p] = true;
       t.dir[t.n] = 1 + 2 * p;
@@ -85,10 +86,11 @@ struct P64 {
       if (t.grp[m] == t.grp[n]) return false;
     return true;
   }
-  static constexpr bool new_base(int n) {
+  static constexpr bool new_base(int n) {          // first / last pair along its primitive vector
     return n == 0 || t.b[n][0] != t.b[n - 1][0] || t.b[n][1] != t.b[n - 1][1] ||
            t.b[n][2] != t.b[n - 1][2];
   }
+  static constexpr bool end_base(int n) { return n + 1 == t.n || new_base(n + 1); }
 };
 static_assert(P64<0, 0>::t.n == 4 && P64<0, 1>::t.n == 4 && P64<0, 2>::t.n == 4 &&
               P64<0, 3>::t.n == 4, "D2Q33 parts");

@@ -16,7 +16,9 @@ struct ModelConst {
   double X2[kMaxGc];   // |xi|^2 = a^2 |e|^2 of each group
   double WX2[kMaxGc];  // W X2
   // with k the gcd of the group's components (e = k b, b primitive):
-  double Wk[kMaxGc];   // W k
+  double Wk[kMaxGc], Wk2[kMaxGc], Wk3[kMaxGc], Wk4[kMaxGc];   // W k, W k^2, ...
+  double WX4[kMaxGc];  // W X2^2
+  float Wlo[kMaxGc], WX2f[kMaxGc], WX2lo[kMaxGc], WX4f[kMaxGc], WX4lo[kMaxGc];   // (hi, lo) pairs
   double X4o8[kMaxGc], kX2o2[kMaxGc], k2X2o4[kMaxGc];   // X2^2 / 8, k X2 / 2, k^2 X2 / 4
   float Wf[kMaxGc];
   float X2f[kMaxGc];
@@ -79,6 +81,8 @@ struct StorageOps {
                            long long ncell, int to_buf, cudaStream_t st);
   // Adjoint (lambda type: FP64 for the FP64 form, FP32 otherwise).
   int adj_elem_bytes;
+  // Blocks of an adjoint step: the length of omega_acc.
+  long long (*adjoint_blocks)(const Grid& g);
   // One reverse step: nu_out = (collision Jacobian)^T lambda_{n+1} with
   // lambda_{n+1}(x, i) = nu_next(x + e_i, i), or dL/drho_N(x) when dldrho != NULL;
   // adds this step's dL/domega block partials into omega_acc[block].
@@ -90,7 +94,7 @@ struct StorageOps {
                            double* d_U, double* d_T, const Grid& g, cudaStream_t st);
 };
 
-// Blocks of the 3D cell launch shared by stream-collide and the adjoint step.
+// Blocks of the 3D cell launch shared by stream-collide and the FP32 adjoint step.
 inline int cell_block_x(int nx) { return nx >= 128 ? 128 : ((nx + 31) / 32) * 32; }
 inline long long cell_blocks(const Grid& g) {
   const int bx = cell_block_x(g.nx);

@@ -5,21 +5,54 @@
 // Adjoint arithmetic type: FP64 for the FP64 form, else FP32.
 using L = std::conditional<std::is_same<S, double>::value, double, float>::type;
 
+// Blocks of an adjoint step (one dL/domega partial each).
+long long adjoint_blocks(const Grid& g) {
+  return std::is_same<S, double>::value ? (g.ncell + 31) / 32 : cell_blocks(g);
+}
+
 // The adjoint kernel for this grid: 32-bit element indices (FP32 adjoint) when
 // Q ncell fits them.
 using AdjointFn = void (*)(const S*, const L*, const double*, L*, double*, Grid, double);
 template <int M, bool kFirst>
 AdjointFn adjoint_kernel(const Grid& g) {
-  if constexpr (std::is_same<L, float>::value) {
-    if ((unsigned long long)Model<M>::Q * (unsigned long long)g.ncell <= 0xFFFFFFFFull)
-      return k_adjoint<M, S, L, kFirst, true>;
-  }
+  if ((unsigned long long)Model<M>::Q * (unsigned long long)g.ncell <= 0xFFFFFFFFull)
+    return k_adjoint<M, S, L, kFirst, true>;
   return k_adjoint<M, S, L, kFirst, false>;
+}
+
+// FP64 form: 32 cells per block, 1, 2 or 4 warps (lin64_warps: the adjoint step has about
+// three times the forward step's instructions in both of its terms).
+template <int M>
+cudaError_t adjoint64_m(const void* state_n, const void* nu_next, const double* dldrho,
+                        void* nu_out, double* omega_acc, const Grid& g, double omega,
+                        cudaStream_t st) {
+  int sms = 0;
+  cudaError_t e = sm_count(&sms);
+  if (e != cudaSuccess) return e;
+  const int w = lin64_warps<M>(g.ncell, sms);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)((g.ncell + 31) / 32));
+  cfg.blockDim = dim3(32 * w);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  auto kern = k_adjoint64<M, false, 1>;
+  if (dldrho) kern = w == 1 ? k_adjoint64<M, true, 1> : w == 2 ? k_adjoint64<M, true, 2> : k_adjoint64<M, true, 4>;
+  else kern = w == 1 ? k_adjoint64<M, false, 1> : w == 2 ? k_adjoint64<M, false, 2> : k_adjoint64<M, false, 4>;
+  return cudaLaunchKernelEx(&cfg, kern, static_cast<const double*>(state_n),
+                            static_cast<const double*>(nu_next), dldrho,
+                            static_cast<double*>(nu_out), omega_acc, g, omega);
 }
 
 template <int M>
 cudaError_t adjoint_m(const void* state_n, const void* nu_next, const double* dldrho, void* nu_out,
                       double* omega_acc, const Grid& g, double omega, cudaStream_t st) {
+  if constexpr (std::is_same<S, double>::value) {
+    return adjoint64_m<M>(state_n, nu_next, dldrho, nu_out, omega_acc, g, omega, st);
+  } else {
   const int bx = cell_block_x(g.nx);
   const dim3 grid((unsigned)((g.nx + bx - 1) / bx), (unsigned)g.ny, (unsigned)g.nz);
   constexpr int smem = adj_smem_bytes<M, L>();
@@ -58,14 +91,15 @@ cudaError_t adjoint_m(const void* state_n, const void* nu_next, const double* dl
   return cudaLaunchKernelEx(&cfg, kern, static_cast<const S*>(state_n),
                             static_cast<const L*>(nu_next), static_cast<const double*>(nullptr),
                             static_cast<L*>(nu_out), omega_acc, g, omega);
+  }
 }
 
 template <int M>
 cudaError_t grad_init_m(const void* nu0, const double* fields, double* d_rho, double* d_U,
                         double* d_T, const Grid& g, cudaStream_t st) {
-  const int bx = cell_block_x(g.nx);
-  const dim3 grid((unsigned)((g.nx + bx - 1) / bx), (unsigned)g.ny, (unsigned)g.nz);
-  k_grad_init<M, L><<<grid, bx, 0, st>>>(static_cast<const L*>(nu0), fields, d_rho, d_U, d_T, g);
+  // blocks of one warp where the FP64 pipe bounds the kernel (see k_stream_collide64)
+  const int bs = std::is_same<L, double>::value ? 32 : 128;
+  k_grad_init<M, L><<<(unsigned)((g.ncell + bs - 1) / bs), bs, 0, st>>>(static_cast<const L*>(nu0), fields, d_rho, d_U, d_T, g);
   return cudaGetLastError();
 }
 

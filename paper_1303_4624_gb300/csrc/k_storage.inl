@@ -319,6 +319,6 @@ cudaError_t set_f(int m, const double* f, void* dst, const Grid& g, cudaStream_t
 
 const StorageOps LBM_OPS = {(int)sizeof(S), upload,       init,      step,         prepare_tma,
                             moments,        get_f,        set_f,     fix_ends,     halo_copy,
-                            (int)sizeof(L), adjoint_step, grad_init};
+                            (int)sizeof(L), adjoint_blocks, adjoint_step, grad_init};
 
 }  // namespace lbm

@@ -201,13 +201,22 @@ bool build_host_model(int model, HostModel* hm) {
     mc.W[g] = hm->W[g];
     mc.X2[g] = a * a * vs.e2[g];
     mc.WX2[g] = mc.W[g] * mc.X2[g];
+    mc.WX4[g] = mc.WX2[g] * mc.X2[g];
     mc.Wf[g] = (float)mc.W[g];
+    mc.Wlo[g] = (float)(mc.W[g] - (double)mc.Wf[g]);
+    mc.WX2f[g] = (float)mc.WX2[g];
+    mc.WX2lo[g] = (float)(mc.WX2[g] - (double)mc.WX2f[g]);
+    mc.WX4f[g] = (float)mc.WX4[g];
+    mc.WX4lo[g] = (float)(mc.WX4[g] - (double)mc.WX4f[g]);
     mc.X2f[g] = (float)mc.X2[g];
     mc.X2lo[g] = (float)(mc.X2[g] - (double)mc.X2f[g]);
   }
   for (int i = 0; i < vs.Q; ++i) {
     const int g = vs.grp[i], k = igcd(igcd(iabs(vs.e[i][0]), iabs(vs.e[i][1])), iabs(vs.e[i][2]));
     mc.Wk[g] = k * mc.W[g];
+    mc.Wk2[g] = k * k * mc.W[g];
+    mc.Wk3[g] = k * k * k * mc.W[g];
+    mc.Wk4[g] = k * k * k * k * mc.W[g];
     mc.X4o8[g] = mc.X2[g] * mc.X2[g] / 8.0;
     mc.kX2o2[g] = k * mc.X2[g] / 2.0;
     mc.k2X2o4[g] = k * k * mc.X2[g] / 4.0;
