@@ -264,13 +264,17 @@ cudaError_t moments_m(const void* src, const Grid& g, double* rho, double* U, do
 
 template <int M>
 cudaError_t get_f_m(const void* src, double* f, const Grid& g, cudaStream_t st) {
-  k_get_f<M, S><<<1024, 256, 0, st>>>(static_cast<const S*>(src), f, g);
+  const long long n = (long long)Model<M>::Q * g.ncell;
+  const auto kern = (reinterpret_cast<uintptr_t>(f) & 15) == 0 ? k_get_f<M, S, true> : k_get_f<M, S, false>;
+  kern<<<(unsigned)((n + kIoRun - 1) / kIoRun), kIoThreads, 0, st>>>(static_cast<const S*>(src), f, g);
   return cudaGetLastError();
 }
 
 template <int M>
 cudaError_t set_f_m(const double* f, void* dst, const Grid& g, cudaStream_t st) {
-  k_set_f<M, S><<<1024, 256, 0, st>>>(f, static_cast<S*>(dst), g);
+  const long long n = (long long)Model<M>::Q * g.ncell;
+  const auto kern = (reinterpret_cast<uintptr_t>(f) & 15) == 0 ? k_set_f<M, S, true> : k_set_f<M, S, false>;
+  kern<<<(unsigned)((n + kIoRun - 1) / kIoRun), kIoThreads, 0, st>>>(f, static_cast<S*>(dst), g);
   return cudaGetLastError();
 }
 

@@ -1308,25 +1308,142 @@ static __global__ void __launch_bounds__(256) k_audit_reduce(const double* __res
 }
 
 // ----------------------------------------------------------------- population I/O (FP64)
-template <int M, class S>
-__global__ void k_get_f(const S* __restrict__ src, double* __restrict__ f, Grid g) {
+// Both kernels are streams of 8 + sizeof(S) bytes an element, and the FP64 pipe is what
+// they must spare: at 64 cycles an FP64 instruction or FP32 / FP64 conversion and
+// scheduler, one such instruction per element already takes as long as the memory
+// traffic of the FP32 form (94.5 M elements, D3Q95 201 x 99 x 50: 163 us against 170).
+// Conversions are therefore done on the integer and FP32 pipes, w (1 + h) is one FMA and
+// f / w - 1 one subtraction (f - w, exact where it cancels) and a product with 1 / w in
+// double-float.  The direction of an element is found by one division per kIoRun
+// elements.  Before: an FP64 division, a 64-bit integer division and two conversions an
+// element, 1771 us (set) and 637 us (get) on that grid.
+constexpr int kIoThreads = 256;
+constexpr int kIoPairs = 8;                          // pairs of elements per thread
+constexpr int kIoRun = kIoThreads * kIoPairs * 2;    // elements per block
+
+// (double)v on the integer pipe (subnormals, Inf and NaN: the conversion instruction).
+__device__ __forceinline__ double widen(float v) {
+  const unsigned u = __float_as_uint(v), m = u & 0x7fffffffu;
+  const bool zero = m == 0;
+  if (!zero && (m < 0x00800000u || m >= 0x7f800000u)) return (double)v;
+  const unsigned hi = (u & 0x80000000u) | (zero ? 0u : (m >> 3) + 0x38000000u);
+  return __hiloint2double((int)hi, (int)(u << 29));
+}
+// d as a double-float pair without the conversion instruction: hi its leading 24 bits
+// (truncated), lo the other 29 rounded to 24.  False (nothing set) outside 2^-63 <= |d| < 2^64.
+__device__ __forceinline__ bool ff_split(double d, FF* v) {
+  const unsigned h = (unsigned)__double2hiint(d), l = (unsigned)__double2loint(d);
+  const unsigned m = h & 0x7fffffffu, e = m >> 20, sign = h & 0x80000000u;
+  if ((m | l) == 0) {
+    *v = {__uint_as_float(sign), 0.f};
+    return true;
+  }
+  if (e < 960u || e >= 1087u) return false;
+  v->hi = __uint_as_float(sign | __funnelshift_l(l, m - 0x38000000u, 3));
+  const float scale = __uint_as_float(sign | ((e - 948u) << 23));   // 2^(e - 1023 - 52)
+  v->lo = __fmul_rn((float)(l & 0x1fffffffu), scale);
+  return true;
+}
+
+// The direction of flat element k and the first element of the next direction.
+struct IoDir {
+  int i;
+  long long next;
+  __device__ __forceinline__ IoDir(long long k, long long ncell) {
+    i = (int)(k / ncell);
+    next = (i + 1) * ncell;
+  }
+  __device__ __forceinline__ int at(long long k, long long ncell) {
+    while (k >= next) {
+      ++i;
+      next += ncell;
+    }
+    return i;
+  }
+};
+
+template <class S>
+struct IoPair {};
+template <>
+struct IoPair<double> { using T = double2; };
+template <>
+struct IoPair<float> { using T = float2; };
+template <>
+struct IoPair<__half> { using T = __half2; };
+template <>
+struct IoPair<__nv_bfloat16> { using T = __nv_bfloat162; };
+
+// VEC: f is 16-byte aligned (a caller's buffer may be aligned to 8 only).
+template <int M, class S, bool VEC>
+__global__ void __launch_bounds__(kIoThreads)
+    k_get_f(const S* __restrict__ src, double* __restrict__ f, Grid g) {
   const ModelConst& mc = c_mc[M];
   const long long n = (long long)Model<M>::Q * g.ncell;
-  for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < n;
-       k += (long long)gridDim.x * blockDim.x) {
-    const int i = (int)(k / g.ncell);
-    f[k] = mc.w[i] * (1.0 + to_double(src[k]));
+  long long k = (long long)blockIdx.x * kIoRun + 2 * threadIdx.x;
+  if (k >= n) return;
+  auto one = [&](S h, int i) {
+    const double w = mc.w[i];
+    if constexpr (std::is_same<S, double>::value) return __fma_rn(w, h, w);
+    else if constexpr (std::is_same<S, float>::value) return __fma_rn(w, widen(h), w);
+    else if constexpr (std::is_same<S, __half>::value) return __fma_rn(w, widen(__half2float(h)), w);
+    else return __fma_rn(w, widen(__bfloat162float(h)), w);
+  };
+  IoDir dir(k, g.ncell);
+#pragma unroll 4
+  for (int j = 0; j < kIoPairs && k < n; ++j, k += 2 * kIoThreads) {
+    if (k + 1 < n) {
+      const typename IoPair<S>::T h = *reinterpret_cast<const typename IoPair<S>::T*>(src + k);
+      const int i0 = dir.at(k, g.ncell), i1 = dir.at(k + 1, g.ncell);
+      const double2 v = make_double2(one(h.x, i0), one(h.y, i1));
+      if constexpr (VEC) {
+        *reinterpret_cast<double2*>(f + k) = v;
+      } else {
+        f[k] = v.x;
+        f[k + 1] = v.y;
+      }
+    } else {
+      f[k] = one(src[k], dir.at(k, g.ncell));
+    }
   }
 }
 
-template <int M, class S>
-__global__ void k_set_f(const double* __restrict__ f, S* __restrict__ dst, Grid g) {
+template <int M, class S, bool VEC>
+__global__ void __launch_bounds__(kIoThreads)
+    k_set_f(const double* __restrict__ f, S* __restrict__ dst, Grid g) {
   const ModelConst& mc = c_mc[M];
   const long long n = (long long)Model<M>::Q * g.ncell;
-  for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < n;
-       k += (long long)gridDim.x * blockDim.x) {
-    const int i = (int)(k / g.ncell);
-    dst[k] = Codec<S>::enc(f[k] / mc.w[i] - 1.0);
+  long long k = (long long)blockIdx.x * kIoRun + 2 * threadIdx.x;
+  if (k >= n) return;
+  auto one = [&](double v, int i) -> S {
+    const double d = __dsub_rn(v, mc.w[i]);
+    if constexpr (std::is_same<S, double>::value) {
+      const double y = __dmul_rn(d, mc.iw[i]);       // and one residual step of d / w
+      const double r = __fma_rn(__fma_rn(-y, mc.w[i], d), mc.iw[i], y);
+      return isfinite(y) ? r : y;                    // (an infinite y has no residual)
+    } else {
+      FF s;
+      if (!ff_split(d, &s)) return Codec<S>::enc(__dmul_rn(d, mc.iw[i]));
+      const float p = __fmul_rn(s.hi, mc.iwf[i]);
+      float e = __fmaf_rn(s.hi, mc.iwf[i], -p);
+      e = __fmaf_rn(s.hi, mc.iwlo[i], e);
+      e = __fmaf_rn(s.lo, mc.iwf[i], e);
+      return ff_round<S>(ff_renorm(p, e));
+    }
+  };
+  IoDir dir(k, g.ncell);
+#pragma unroll 4
+  for (int j = 0; j < kIoPairs && k < n; ++j, k += 2 * kIoThreads) {
+    if (k + 1 < n) {
+      double2 v;
+      if constexpr (VEC) v = *reinterpret_cast<const double2*>(f + k);
+      else v = make_double2(f[k], f[k + 1]);
+      typename IoPair<S>::T h;
+      h.x = one(v.x, dir.at(k, g.ncell));
+      h.y = one(v.y, dir.at(k + 1, g.ncell));
+      *reinterpret_cast<typename IoPair<S>::T*>(dst + k) = h;
+    } else {
+      dst[k] = one(f[k], dir.at(k, g.ncell));
+    }
   }
 }
 

@@ -221,6 +221,9 @@ bool build_host_model(int model, HostModel* hm) {
     mc.kX2o2[g] = k * mc.X2[g] / 2.0;
     mc.k2X2o4[g] = k * k * mc.X2[g] / 4.0;
     mc.w[i] = hm->w[i];
+    mc.iw[i] = 1.0 / hm->w[i];
+    mc.iwf[i] = (float)mc.iw[i];
+    mc.iwlo[i] = (float)(mc.iw[i] - (double)mc.iwf[i]);
     for (int d = 0; d < 3; ++d) {
       mc.e[i][d] = vs.e[i][d];
       mc.ef[i][d] = (float)vs.e[i][d];
