@@ -24,8 +24,8 @@ struct ModelConst {
   float X2f[kMaxGc];
   float X2lo[kMaxGc];  // X2 - X2f: with X2f, X2 as a double-float (hi, lo) pair
   double w[kMaxQc];    // weight per direction (storage order)
-  double iw[kMaxQc];   // 1 / w, and the same as a double-float (hi, lo) pair
-  float iwf[kMaxQc], iwlo[kMaxQc];
+  double iw[kMaxQc], iw2[kMaxQc];   // 1 / w rounded, and the rest of it
+  float iwf[kMaxQc], iwlo[kMaxQc];  // 1 / w as a double-float (hi, lo) pair
   double a;            // sqrt(2) c: xi_i = a e_i
   float af, alo;       // a rounded to FP32, and a - af
   double c;

@@ -1315,17 +1315,24 @@ static __global__ void __launch_bounds__(256) k_audit_reduce(const double* __res
 // Conversions are therefore done on the integer and FP32 pipes, w (1 + h) is one FMA and
 // f / w - 1 one subtraction (f - w, exact where it cancels) and a product with 1 / w in
 // double-float.  The direction of an element is found by one division per kIoRun
-// elements.  Before: an FP64 division, a 64-bit integer division and two conversions an
-// element, 1771 us (set) and 637 us (get) on that grid.
+// elements.  With an FP64 division, a 64-bit integer division and two conversions an
+// element set took 1771 us and get 637 us on that grid; now 207 and 198 us.
 constexpr int kIoThreads = 256;
 constexpr int kIoPairs = 8;                          // pairs of elements per thread
 constexpr int kIoRun = kIoThreads * kIoPairs * 2;    // elements per block
 
+// The rare cases are calls: as an inline branch the compiler predicates their FP64
+// instructions, which then take their 64 cycles for every element all the same.
+static __device__ __noinline__ double widen_any(float v) { return (double)v; }
+template <class S>
+static __device__ __noinline__ S enc_any(double d, double iw) {
+  return Codec<S>::enc(__dmul_rn(d, iw));
+}
 // (double)v on the integer pipe (subnormals, Inf and NaN: the conversion instruction).
 __device__ __forceinline__ double widen(float v) {
   const unsigned u = __float_as_uint(v), m = u & 0x7fffffffu;
   const bool zero = m == 0;
-  if (!zero && (m < 0x00800000u || m >= 0x7f800000u)) return (double)v;
+  if (!zero && (m < 0x00800000u || m >= 0x7f800000u)) return widen_any(v);
   const unsigned hi = (u & 0x80000000u) | (zero ? 0u : (m >> 3) + 0x38000000u);
   return __hiloint2double((int)hi, (int)(u << 29));
 }
@@ -1345,20 +1352,32 @@ __device__ __forceinline__ bool ff_split(double d, FF* v) {
   return true;
 }
 
-// The direction of flat element k and the first element of the next direction.
-struct IoDir {
+// The weight of flat element k's direction, kept in registers until an element of another
+// direction comes.
+struct IoWeight {
   int i;
-  long long next;
-  __device__ __forceinline__ IoDir(long long k, long long ncell) {
+  long long next;            // first element of the next direction
+  double w, iw, iw2;
+  float iwf, iwlo;
+  __device__ __forceinline__ IoWeight(const ModelConst& mc, long long k, long long ncell) {
     i = (int)(k / ncell);
     next = (i + 1) * ncell;
+    load(mc);
   }
-  __device__ __forceinline__ int at(long long k, long long ncell) {
-    while (k >= next) {
+  __device__ __forceinline__ void load(const ModelConst& mc) {
+    w = mc.w[i];
+    iw = mc.iw[i];
+    iw2 = mc.iw2[i];
+    iwf = mc.iwf[i];
+    iwlo = mc.iwlo[i];
+  }
+  __device__ __forceinline__ void advance(const ModelConst& mc, long long k, long long ncell) {
+    if (k < next) return;
+    do {
       ++i;
       next += ncell;
-    }
-    return i;
+    } while (k >= next);
+    load(mc);
   }
 };
 
@@ -1381,20 +1400,23 @@ __global__ void __launch_bounds__(kIoThreads)
   const long long n = (long long)Model<M>::Q * g.ncell;
   long long k = (long long)blockIdx.x * kIoRun + 2 * threadIdx.x;
   if (k >= n) return;
-  auto one = [&](S h, int i) {
-    const double w = mc.w[i];
+  auto one = [&](S h, double w) {
     if constexpr (std::is_same<S, double>::value) return __fma_rn(w, h, w);
     else if constexpr (std::is_same<S, float>::value) return __fma_rn(w, widen(h), w);
     else if constexpr (std::is_same<S, __half>::value) return __fma_rn(w, widen(__half2float(h)), w);
     else return __fma_rn(w, widen(__bfloat162float(h)), w);
   };
-  IoDir dir(k, g.ncell);
-#pragma unroll 4
-  for (int j = 0; j < kIoPairs && k < n; ++j, k += 2 * kIoThreads) {
+  IoWeight wt(mc, k, g.ncell);
+#pragma unroll
+  for (int j = 0; j < kIoPairs; ++j, k += 2 * kIoThreads) {
+    if (k >= n) break;
+    wt.advance(mc, k, g.ncell);
     if (k + 1 < n) {
       const typename IoPair<S>::T h = *reinterpret_cast<const typename IoPair<S>::T*>(src + k);
-      const int i0 = dir.at(k, g.ncell), i1 = dir.at(k + 1, g.ncell);
-      const double2 v = make_double2(one(h.x, i0), one(h.y, i1));
+      double2 v;
+      v.x = one(h.x, wt.w);
+      wt.advance(mc, k + 1, g.ncell);
+      v.y = one(h.y, wt.w);
       if constexpr (VEC) {
         *reinterpret_cast<double2*>(f + k) = v;
       } else {
@@ -1402,7 +1424,7 @@ __global__ void __launch_bounds__(kIoThreads)
         f[k + 1] = v.y;
       }
     } else {
-      f[k] = one(src[k], dir.at(k, g.ncell));
+      f[k] = one(src[k], wt.w);
     }
   }
 }
@@ -1414,35 +1436,39 @@ __global__ void __launch_bounds__(kIoThreads)
   const long long n = (long long)Model<M>::Q * g.ncell;
   long long k = (long long)blockIdx.x * kIoRun + 2 * threadIdx.x;
   if (k >= n) return;
-  auto one = [&](double v, int i) -> S {
-    const double d = __dsub_rn(v, mc.w[i]);
+  auto one = [&](double v, const IoWeight& q) -> S {
     if constexpr (std::is_same<S, double>::value) {
-      const double y = __dmul_rn(d, mc.iw[i]);       // and one residual step of d / w
-      const double r = __fma_rn(__fma_rn(-y, mc.w[i], d), mc.iw[i], y);
-      return isfinite(y) ? r : y;                    // (an infinite y has no residual)
+      // v / w - 1 with 1 / w = iw + iw2: half an ulp of 1, as the division and the
+      // subtraction had, in two FMAs (Inf and NaN as they are)
+      if ((__double2hiint(v) & 0x7ff00000) == 0x7ff00000) return v;
+      return __fma_rn(v, q.iw, __fma_rn(v, q.iw2, -1.0));
     } else {
+      const double d = __dsub_rn(v, q.w);
       FF s;
-      if (!ff_split(d, &s)) return Codec<S>::enc(__dmul_rn(d, mc.iw[i]));
-      const float p = __fmul_rn(s.hi, mc.iwf[i]);
-      float e = __fmaf_rn(s.hi, mc.iwf[i], -p);
-      e = __fmaf_rn(s.hi, mc.iwlo[i], e);
-      e = __fmaf_rn(s.lo, mc.iwf[i], e);
+      if (!ff_split(d, &s)) return enc_any<S>(d, q.iw);
+      const float p = __fmul_rn(s.hi, q.iwf);
+      float e = __fmaf_rn(s.hi, q.iwf, -p);
+      e = __fmaf_rn(s.hi, q.iwlo, e);
+      e = __fmaf_rn(s.lo, q.iwf, e);
       return ff_round<S>(ff_renorm(p, e));
     }
   };
-  IoDir dir(k, g.ncell);
-#pragma unroll 4
-  for (int j = 0; j < kIoPairs && k < n; ++j, k += 2 * kIoThreads) {
+  IoWeight wt(mc, k, g.ncell);
+#pragma unroll
+  for (int j = 0; j < kIoPairs; ++j, k += 2 * kIoThreads) {
+    if (k >= n) break;
+    wt.advance(mc, k, g.ncell);
     if (k + 1 < n) {
       double2 v;
       if constexpr (VEC) v = *reinterpret_cast<const double2*>(f + k);
       else v = make_double2(f[k], f[k + 1]);
       typename IoPair<S>::T h;
-      h.x = one(v.x, dir.at(k, g.ncell));
-      h.y = one(v.y, dir.at(k + 1, g.ncell));
+      h.x = one(v.x, wt);
+      wt.advance(mc, k + 1, g.ncell);
+      h.y = one(v.y, wt);
       *reinterpret_cast<typename IoPair<S>::T*>(dst + k) = h;
     } else {
-      dst[k] = one(f[k], dir.at(k, g.ncell));
+      dst[k] = one(f[k], wt);
     }
   }
 }
