@@ -12,28 +12,29 @@ constexpr int kMaxGc = 10;
 
 // Per-model constants solved on the host (Formula 5) and kept in constant memory.
 struct ModelConst {
-  double W[kMaxGc];    // weight of each symmetry group
-  double X2[kMaxGc];   // |xi|^2 = a^2 |e|^2 of each group
-  double WX2[kMaxGc];  // W X2
-  // with k the gcd of the group's components (e = k b, b primitive):
-  double Wk[kMaxGc], Wk2[kMaxGc], Wk3[kMaxGc], Wk4[kMaxGc];   // W k, W k^2, ...
-  double WX4[kMaxGc];  // W X2^2
-  float Wlo[kMaxGc], WX2f[kMaxGc], WX2lo[kMaxGc], WX4f[kMaxGc], WX4lo[kMaxGc];   // (hi, lo) pairs
-  double X4o8[kMaxGc], kX2o2[kMaxGc], k2X2o4[kMaxGc];   // X2^2 / 8, k X2 / 2, k^2 X2 / 4
-  float Wf[kMaxGc];
-  float X2f[kMaxGc];
+  // read by the FP32-arithmetic kernels
+  float Wf[kMaxGc];    // weight of each symmetry group
+  float X2f[kMaxGc];   // |xi|^2 = a^2 |e|^2 of each group
   float X2lo[kMaxGc];  // X2 - X2f: with X2f, X2 as a double-float (hi, lo) pair
-  double w[kMaxQc];    // weight per direction (storage order)
-  double iw[kMaxQc], iw2[kMaxQc];   // 1 / w rounded, and the rest of it
-  float iwf[kMaxQc], iwlo[kMaxQc];  // 1 / w as a double-float (hi, lo) pair
-  double a;            // sqrt(2) c: xi_i = a e_i
   float af, alo;       // a rounded to FP32, and a - af
-  double c;
-  double T0;           // 1 / (2 c^2), lattice units
   float T0f, iT0f;     // T0 and 1 / T0 rounded to FP32
   float iT0lo;         // 1 / T0 - iT0f
-  int e[kMaxQc][3];    // lattice vectors in storage order (zero-padded to 3 components)
-  float ef[kMaxQc][3]; // the same as FP32 (loops that index directions at run time)
+  float Wlo[kMaxGc], WX2f[kMaxGc], WX2lo[kMaxGc], WX4f[kMaxGc], WX4lo[kMaxGc];   // (hi, lo) pairs
+  float ef[kMaxQc][3]; // lattice vectors (loops that index directions at run time)
+  // the FP64 form
+  double W[kMaxGc], X2[kMaxGc];
+  double WX2[kMaxGc], WX4[kMaxGc];   // W X2, W X2^2
+  // with k the gcd of the group's components (e = k b, b primitive):
+  double Wk[kMaxGc], Wk2[kMaxGc], Wk3[kMaxGc], Wk4[kMaxGc];   // W k, W k^2, ...
+  double X4o8[kMaxGc], kX2o2[kMaxGc], k2X2o4[kMaxGc];   // X2^2 / 8, k X2 / 2, k^2 X2 / 4
+  double a;            // sqrt(2) c: xi_i = a e_i
+  double c;
+  double T0;           // 1 / (2 c^2), lattice units
+  // per direction (storage order)
+  double w[kMaxQc];                 // weight
+  double iw[kMaxQc], iw2[kMaxQc];   // 1 / w rounded, and the rest of it
+  float iwf[kMaxQc], iwlo[kMaxQc];  // 1 / w as a double-float (hi, lo) pair
+  int e[kMaxQc][3];                 // lattice vectors (zero-padded to 3 components)
 };
 
 struct Grid {
