@@ -49,6 +49,15 @@ struct StepTest {
   unsigned long long limit_ns;
 };
 
+// Fixed end planes (the shock tube's end conditions): the cells with coordinate < width
+// (side 0) or >= N - width (side 1) along `axis` (0 x, 1 y, 2 z) hold the populations of
+// template cell `side`; tmpl is [Q][2] in the storage type.
+struct Ends {
+  int axis, width;
+  const void* tmpl;
+};
+constexpr Ends kNoEnds = {0, 0, nullptr};
+
 // Launchers of one storage form (one translation unit each).  All enqueue on
 // `st` and return the launch status.
 struct StorageOps {
@@ -57,13 +66,15 @@ struct StorageOps {
   // The equilibrium of the fields for cells [begin, end) (U strided by g.ncell).
   cudaError_t (*init)(int model, const double* rho, const double* U, const double* T, void* dst,
                       const Grid& g, long long begin, long long end, cudaStream_t st);
-  // One stream-collide step.  variant: kVariantDirect, kVariantTma, kVariantSplit or
+  // One stream-collide step.  ends: the fixed end planes, written by the same launch (direct
+  // variant only; width 0: none).  variant: kVariantDirect, kVariantTma, kVariantSplit or
   // kVariantPair, or-ed with kStepReverse for the direct and pair kernels (the caller
   // checks applicability: Nx % 8 == 0 for TMA, Nx even and 16-bit storage for pair).  status: device int
   // set to 1 if a TMA launch gave up waiting for its copies.  test: NULL, or the
   // failure-detection test setting of a TMA launch (see StepTest).
   cudaError_t (*step)(int model, const void* src, void* dst, const Grid& g, double omega,
-                      int variant, int* status, const StepTest* test, cudaStream_t st);
+                      int variant, int* status, const StepTest* test, const Ends& ends,
+                      cudaStream_t st);
   // One-time per-device launch set-up of the TMA kernels (shared-memory opt-in and
   // occupancy), done before any stream capture.
   cudaError_t (*prepare_tma)(int model);

@@ -167,6 +167,23 @@ DirectFn direct_kernel(const Grid& g, int rev) {
   return rev ? k_stream_collide<M, S, true, false> : k_stream_collide<M, S, false, false>;
 }
 
+// The linear-index kernel: 32-bit element indices for D3Q95 FP32 where they fit.
+using LinearFn = void (*)(const S*, S*, Grid, double, Ends);
+template <int M, bool NARROW>
+LinearFn linear_kernel_n(int rev, bool ends) {
+  if (ends)
+    return rev ? k_stream_collide_linear<M, S, true, NARROW, true> : k_stream_collide_linear<M, S, false, NARROW, true>;
+  return rev ? k_stream_collide_linear<M, S, true, NARROW, false> : k_stream_collide_linear<M, S, false, NARROW, false>;
+}
+template <int M>
+LinearFn linear_kernel(const Grid& g, int rev, bool ends) {
+  if constexpr (DirectNarrow<M, S>::value) {
+    if ((unsigned long long)Model<M>::Q * (unsigned long long)g.ncell <= 0xFFFFFFFFull)
+      return linear_kernel_n<M, true>(rev, ends);
+  }
+  return linear_kernel_n<M, false>(rev, ends);
+}
+
 // SMs of the current device (looked up once per device).
 cudaError_t sm_count(int* sms) {
   static std::atomic<int> known[16];
@@ -186,7 +203,7 @@ cudaError_t sm_count(int* sms) {
 // The FP64 kernel: 32 cells per block, 1, 2 or 4 warps (lin64_warps).
 template <int M>
 cudaError_t step64_m(const void* src, void* dst, const Grid& g, double omega, int rev,
-                     cudaStream_t st) {
+                     const Ends& ends, cudaStream_t st) {
   int sms = 0;
   cudaError_t e = sm_count(&sms);
   if (e != cudaSuccess) return e;
@@ -205,12 +222,12 @@ cudaError_t step64_m(const void* src, void* dst, const Grid& g, double omega, in
   else if (w == 2) kern = k_stream_collide64<M, false, 2>;
   else kern = k_stream_collide64<M, false, 4>;
   return cudaLaunchKernelEx(&cfg, kern, static_cast<const double*>(src), static_cast<double*>(dst),
-                            g, omega);
+                            g, omega, ends);
 }
 
 template <int M>
 cudaError_t step_m(const void* src, void* dst, const Grid& g, double omega, int variant, int* status,
-                   const StepTest* test, cudaStream_t st) {
+                   const StepTest* test, const Ends& ends, cudaStream_t st) {
   const int rev = (variant & kStepReverse) ? 1 : 0;
   variant &= ~kStepReverse;
   if (variant == kVariantTma) return step_tma_m<M>(src, dst, g, omega, status, test, st);
@@ -227,28 +244,26 @@ cudaError_t step_m(const void* src, void* dst, const Grid& g, double omega, int 
     }
   }
   if constexpr (std::is_same<S, double>::value) {
-    return step64_m<M>(src, dst, g, omega, rev, st);
+    return step64_m<M>(src, dst, g, omega, rev, ends, st);
   } else {
-  const int bx = cell_block_x(g.nx);
-  const dim3 grid((unsigned)((g.nx + bx - 1) / bx), (unsigned)g.ny, (unsigned)g.nz);
-#ifndef LBM_NO_PDL
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = dim3(bx);
-  cfg.dynamicSmemBytes = 0;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, direct_kernel<M>(g, rev), static_cast<const S*>(src),
-                            static_cast<S*>(dst), g, omega);
-#else
-  direct_kernel<M>(g, rev)<<<grid, bx, 0, st>>>(static_cast<const S*>(src), static_cast<S*>(dst), g,
-                                                omega);
-  return cudaGetLastError();
-#endif
+    cudaLaunchConfig_t cfg = {};
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (ends.width > 0 || linear_rows<M, S>(g)) {
+      cfg.gridDim = dim3((unsigned)((g.ncell + kLinThreads - 1) / kLinThreads));
+      cfg.blockDim = dim3(kLinThreads);
+      return cudaLaunchKernelEx(&cfg, linear_kernel<M>(g, rev, ends.width > 0),
+                                static_cast<const S*>(src), static_cast<S*>(dst), g, omega, ends);
+    }
+    const int bx = cell_block_x(g.nx);
+    cfg.gridDim = dim3((unsigned)((g.nx + bx - 1) / bx), (unsigned)g.ny, (unsigned)g.nz);
+    cfg.blockDim = dim3(bx);
+    return cudaLaunchKernelEx(&cfg, direct_kernel<M>(g, rev), static_cast<const S*>(src),
+                              static_cast<S*>(dst), g, omega);
   }
 }
 
@@ -303,9 +318,9 @@ cudaError_t init(int m, const double* rho, const double* U, const double* T, voi
                 : init_m<1>(rho, U, T, dst, g, begin, end, st);
 }
 cudaError_t step(int m, const void* src, void* dst, const Grid& g, double omega, int variant,
-                 int* status, const StepTest* test, cudaStream_t st) {
-  return m == 0 ? step_m<0>(src, dst, g, omega, variant, status, test, st)
-                : step_m<1>(src, dst, g, omega, variant, status, test, st);
+                 int* status, const StepTest* test, const Ends& ends, cudaStream_t st) {
+  return m == 0 ? step_m<0>(src, dst, g, omega, variant, status, test, ends, st)
+                : step_m<1>(src, dst, g, omega, variant, status, test, ends, st);
 }
 cudaError_t moments(int m, const void* src, const Grid& g, double* rho, double* U, double* T,
                     double* partials, long long block0, long long nblocks, cudaStream_t st) {

@@ -679,6 +679,79 @@ __global__ void __launch_bounds__(128, DirectMinBlocks<M, S>::value)
   }
 }
 
+// Linear-index direct kernel: thread t of the grid updates cell t, so rows of any length
+// fill the warps, and a warp's stores are aligned whatever Nx.  The row-mapped kernel above
+// leaves lanes idle in the last block of each row and in its last warp (11 of 32 used for
+// Nx = 11, 201 of 256 for Nx = 201) and starts odd rows off the sector boundaries, but
+// keeps the y and z offsets uniform in a block (see linear_rows for the rule between the
+// two).  Same arithmetic, same bits.
+// ENDS: the fixed end planes are written here as well (a cell of an end plane stores its
+// template and gathers nothing) instead of by a second kernel after the step.
+// In y and z only the offsets that occur are formed; lanes of a warp differ in them.
+#ifndef LBM_LIN_THREADS
+#define LBM_LIN_THREADS 128
+#endif
+constexpr int kLinThreads = LBM_LIN_THREADS;
+template <int M, class S, bool REV, bool NARROW, bool ENDS>
+__global__ void __launch_bounds__(kLinThreads, DirectMinBlocks<M, S>::value * 128 / kLinThreads)
+    k_stream_collide_linear(const S* __restrict__ src, S* __restrict__ dst, Grid g, double omega,
+                            Ends ends) {
+  using Mo = Model<M>;
+  constexpr int D = Mo::D, RR = Mo::R;
+  wait_prior_grid();
+  allow_next_grid();
+  const unsigned b = REV ? gridDim.x - 1 - blockIdx.x : blockIdx.x;
+  const uint32_t cell = b * kLinThreads + threadIdx.x;
+  if (cell >= (uint32_t)g.ncell) return;
+  const uint32_t row = cell / (uint32_t)g.nx;
+  const int x = (int)(cell - row * (uint32_t)g.nx);
+  const int z = D == 3 ? (int)(row / (uint32_t)g.ny) : 0;
+  const int y = (int)row - z * g.ny;
+  if constexpr (ENDS) {
+    const int c = ends.axis == 0 ? x : (ends.axis == 1 ? y : z);
+    const int n = ends.axis == 0 ? g.nx : (ends.axis == 1 ? g.ny : g.nz);
+    if (c < ends.width || c >= n - ends.width) {
+      const S* t = static_cast<const S*>(ends.tmpl) + (c < ends.width ? 0 : 1);
+#pragma unroll 8
+      for (int i = 0; i < Mo::Q; ++i) dst[(size_t)i * (size_t)g.ncell + cell] = __ldg(t + 2 * i);
+      return;
+    }
+  }
+  int xo[2 * RR + 1], yo[2 * RR + 1], zo[2 * RR + 1];
+  neighbour_offsets<D, RR>(x, y, z, g.nx, g.ny, g.nz, g.nxy, xo, yo, zo);
+  using Index = typename std::conditional<NARROW, uint32_t, size_t>::type;
+  const Index nc = (Index)g.ncell;
+  cell_update<M, S>(
+      [&](auto I) {
+        constexpr int i = decltype(I)::value;
+        constexpr int ex = Mo::vs.e[i][0], ey = Mo::vs.e[i][1], ez = Mo::vs.e[i][2];
+        return Codec<S>::ld(src + (Index)((Index)i * nc + (Index)(zo[ez + RR] + yo[ey + RR] + xo[ex + RR])));
+      },
+      omega,
+      [&](auto I, typename Codec<S>::R v) {
+        Codec<S>::st(dst + (Index)((Index)decltype(I)::value * nc + cell), v);
+      });
+}
+
+// Row-mapped or linear.  Measured (us a step, rows / linear, D3Q95 FP32 unless named): idle
+// lanes cost the row mapping, 11x11x800 25.9 / 12.0, 72x64x64 42.7 / 37.4, 168x64x64 93.0 /
+// 84.2, 201x99x50 146 / 132; without them its uniform offsets win, 128x128x128 236 / 245,
+// 248x64x64 (3 % idle) 121 / 126, so the line is drawn at one idle lane in 16.  Rows that
+// start off the 32-byte sectors cost partial sector writes once the state leaves L2:
+// 250x64x64 131 / 125, D2Q33 2046x1024 90.1 / 82.7, but D2Q33 1021x515 (two copies of 69 MB)
+// 22.3 / 22.6.
+template <int M, class S>
+inline bool linear_rows(const Grid& g) {
+#ifdef LBM_LIN_ALWAYS
+  return LBM_LIN_ALWAYS;
+#endif
+  const int bx = cell_block_x(g.nx);
+  const long long padded = (long long)(g.nx + bx - 1) / bx * bx;
+  if (padded * 16 > (long long)g.nx * 17) return true;
+  return g.nx * sizeof(S) % 32 != 0 &&
+         (size_t)Model<M>::Q * (size_t)g.ncell * sizeof(S) > ((size_t)128 << 20);
+}
+
 // FP64 form: linear cell index (rows of any length fill the warps), 32 cells per block,
 // WARPS warps per block.  The FP64 pipe bounds the form (see collide64.cuh): each of an
 // SM's four schedulers takes 64 cycles an FP64 instruction, so the grid's time is that of
@@ -699,7 +772,7 @@ __device__ __forceinline__ double ld_again(const double* p) {
 template <int M, bool REV, int WARPS>
 __global__ void __launch_bounds__(32 * WARPS, 8 / WARPS)
     k_stream_collide64(const double* __restrict__ src, double* __restrict__ dst, Grid g,
-                       double omega) {
+                       double omega, Ends ends) {
   using Mo = Model<M>;
   constexpr int D = Mo::D, RR = Mo::R;
   constexpr std::integral_constant<int, 0> rest{};
@@ -722,8 +795,14 @@ __global__ void __launch_bounds__(32 * WARPS, 8 / WARPS)
     constexpr int ex = Mo::vs.e[i][0], ey = Mo::vs.e[i][1], ez = Mo::vs.e[i][2];
     return src + (size_t)i * (size_t)g.ncell + (zo[ez + RR] + yo[ey + RR] + xo[ex + RR]);
   };
+  // fixed end planes (width 0: none): a cell there takes its template's populations
+  const int c_ax = ends.axis == 0 ? x : (ends.axis == 1 ? y : z);
+  const int n_ax = ends.axis == 0 ? g.nx : (ends.axis == 1 ? g.ny : g.nz);
+  const bool low = c_ax < ends.width, fixed = low || c_ax >= n_ax - ends.width;
+  const double* tmpl = static_cast<const double*>(ends.tmpl) + (low ? 0 : 1);
   auto st = [&](auto I, double v) {
-    if (active) dst[(size_t)decltype(I)::value * (size_t)g.ncell + cell] = v;
+    constexpr int i = decltype(I)::value;
+    if (active) dst[(size_t)i * (size_t)g.ncell + cell] = fixed ? __ldg(tmpl + 2 * i) : v;
   };
   auto hm = [&](auto I) { return __ldg(at(I)); };
   auto hr = [&](auto I) { return ld_again(at(I)); };
@@ -1314,7 +1393,7 @@ static __global__ void __launch_bounds__(256) k_audit_reduce(const double* __res
 // traffic of the FP32 form (94.5 M elements, D3Q95 201 x 99 x 50: 163 us against 170).
 // Conversions are therefore done on the integer and FP32 pipes, w (1 + h) is one FMA and
 // f / w - 1 one subtraction (f - w, exact where it cancels) and a product with 1 / w in
-// double-float.  The direction of an element is found by one division per kIoRun
+// double-float, rounded as the FP64 division and subtraction round.  The direction of an element is found by one division per kIoRun
 // elements.  With an FP64 division, a 64-bit integer division and two conversions an
 // element set took 1771 us and get 637 us on that grid; now 207 and 198 us.
 constexpr int kIoThreads = 256;
@@ -1325,8 +1404,8 @@ constexpr int kIoRun = kIoThreads * kIoPairs * 2;    // elements per block
 // instructions, which then take their 64 cycles for every element all the same.
 static __device__ __noinline__ double widen_any(float v) { return (double)v; }
 template <class S>
-static __device__ __noinline__ S enc_any(double d, double iw) {
-  return Codec<S>::enc(__dmul_rn(d, iw));
+static __device__ __noinline__ S enc_any(double f, double w) {
+  return Codec<S>::enc(f / w - 1.0);
 }
 // (double)v on the integer pipe (subnormals, Inf and NaN: the conversion instruction).
 __device__ __forceinline__ double widen(float v) {
@@ -1445,12 +1524,23 @@ __global__ void __launch_bounds__(kIoThreads)
     } else {
       const double d = __dsub_rn(v, q.w);
       FF s;
-      if (!ff_split(d, &s)) return enc_any<S>(d, q.iw);
+      if (!ff_split(d, &s)) return enc_any<S>(v, q.w);
       const float p = __fmul_rn(s.hi, q.iwf);
       float e = __fmaf_rn(s.hi, q.iwf, -p);
       e = __fmaf_rn(s.hi, q.iwlo, e);
       e = __fmaf_rn(s.lo, q.iwf, e);
-      return ff_round<S>(ff_renorm(p, e));
+      const FF h = ff_renorm(p, e);
+      if constexpr (sizeof(S) == 4) {
+        // next to a midpoint of two FP32 values (within 2^-18 of half an ulp, which covers
+        // the double-float error and FP64's own 2^-53 of f / w for |h| above 1e-3; closer
+        // in proportion below), or at a power of two, the FP64 sequence decides the rounding
+        const unsigned u = __float_as_uint(h.hi);
+        const float half_ulp = __uint_as_float((u & 0x7f800000u) - (24u << 23));
+        const float tol = __fmaf_rn(half_ulp, 0x1p-18f, 0x1p-52f * (1.0f + fabsf(h.hi)));
+        if (h.hi != 0.f && (fabsf(fabsf(h.lo) - half_ulp) <= tol || (u & 0x007fffffu) == 0))
+          return enc_any<S>(v, q.w);
+      }
+      return ff_round<S>(h);
     }
   };
   IoWeight wt(mc, k, g.ncell);

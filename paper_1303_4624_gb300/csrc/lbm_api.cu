@@ -483,11 +483,14 @@ cudaError_t enqueue_steps(lbm_ctx* c, int64_t n, int variant, int* cur, cudaStre
       t = &c->test;
       c->test_pending = false;
     }
+    // the direct kernels write the fixed end planes themselves
+    const bool fused = c->fix_width > 0 && variant == kVariantDirect;
+    const Ends ends = fused ? Ends{c->fix_axis, c->fix_width, c->fix_tmpl.p} : kNoEnds;
     cudaError_t e = c->ops->step(c->model, c->state[*cur].p, c->state[*cur ^ 1].p, c->g, c->omega,
-                                 v, static_cast<int*>(c->status.p), t, st);
+                                 v, static_cast<int*>(c->status.p), t, ends, st);
     if (e != cudaSuccess) return e;
     *cur ^= 1;
-    if (c->fix_width > 0) {
+    if (c->fix_width > 0 && !fused) {
       e = c->ops->fix_ends(c->state[*cur].p, c->g, c->fix_axis, c->fix_width, c->fix_tmpl.p, c->Q,
                            st);
       if (e != cudaSuccess) return e;
@@ -531,7 +534,7 @@ bool capture_steps(lbm_ctx* c, int parity, int variant) {
 
 int do_steps(lbm_ctx* c, int64_t n) {
   const int variant = pick_variant(c);
-  const int64_t per_step = c->fix_width > 0 ? 2 : 1;
+  const int64_t per_step = c->fix_width > 0 && variant != kVariantDirect ? 2 : 1;
   int64_t done = 0;
   if (c->graph_steps > 0 && !c->test_pending && n >= 2 * c->graph_steps &&
       (c->graph.exec[c->cur] || capture_steps(c, c->cur, variant))) {
