@@ -42,21 +42,6 @@ struct EqGrad {
 };
 
 
-// Pairs [first, end) of symmetry group g (g >= 1) in storage order.
-template <int M>
-struct ShellPairs {
-  static constexpr int first(int g) {
-    int p = 0;
-    while (p < Model<M>::NP && Model<M>::vs.grp[1 + 2 * p] != g) ++p;
-    return p;
-  }
-  static constexpr int end(int g) {
-    int p = first(g);
-    while (p < Model<M>::NP && Model<M>::vs.grp[1 + 2 * p] == g) ++p;
-    return p;
-  }
-};
-
 // Passes 2 and 3 as loops over each shell's pairs (lattice vectors read from
 // constant memory) instead of fully unrolled over all pairs: a smaller kernel for
 // the instruction cache.  Needs lambda in shared memory or uniform (FP32 adjoint).
@@ -385,8 +370,7 @@ __global__ void __launch_bounds__(kAdjThreads, AdjMinBlocks<S>::value)
 // instructions counted (see collide64.cuh and contract.cuh): the forward moments shell by
 // shell, the contractions once per primitive vector; ~600 FP64 operations a D2Q33 cell
 // against ~900 pair by pair.  Linear cell index, 32 cells per block, shared by WARPS = 1, 2
-// or 4 warps as in k_stream_collide64.  State and lambda are read again where they are used
-// again; the FP64 pipe bounds the kernel and memory has the time.
+// or 4 warps as in k_stream_collide64.
 template <int M, bool kFirst, int WARPS>
 __global__ void __launch_bounds__(32 * WARPS, 8 / WARPS)
     k_adjoint64(const double* __restrict__ state, const double* __restrict__ nu_next,
@@ -414,11 +398,23 @@ __global__ void __launch_bounds__(32 * WARPS, 8 / WARPS)
     return __ldg(state + (size_t)i * nc + (zo[ez + RR] + yo[ey + RR] + xo[ex + RR]));
   };
   const double l1 = kFirst ? dldrho[at0] : 0.0;
-  auto lam = [&](auto I) -> double {       // nu_next(x + e_i, i)
-    constexpr int i = decltype(I)::value;
-    constexpr int ex = Mo::vs.e[i][0], ey = Mo::vs.e[i][1], ez = Mo::vs.e[i][2];
+  // lambda_i = nu_next(x + e_i, i), used three times: kept in shared memory (each thread its
+  // own copies, of its warp's directions)
+  extern __shared__ __align__(16) double stage64[];
+  double* const mine = stage64 + lane;
+  if constexpr (!kFirst) {
+    sfor<0, Mo::Q>([&](auto I) {
+      constexpr int i = decltype(I)::value;
+      constexpr int ex = Mo::vs.e[i][0], ey = Mo::vs.e[i][1], ez = Mo::vs.e[i][2];
+      constexpr int p = i == 0 ? -1 : shell_part64<M>(Mo::vs.grp[i]);
+      if (WARPS == 1 || i == 0 || p / PW == warp)
+        cp_async8(mine + 32 * i, nu_next + (size_t)i * nc + (zo[RR - ez] + yo[RR - ey] + xo[RR - ex]));
+    });
+    cp_async_wait_all();
+  }
+  auto lam = [&](auto I) -> double {
     if constexpr (kFirst) return l1;
-    else return ld_again(nu_next + (size_t)i * nc + (zo[RR - ez] + yo[RR - ey] + xo[RR - ex]));
+    else return mine[32 * decltype(I)::value];
   };
   __shared__ double xch[WARPS][7][32];
   // sums over the warps, in order; the value of warp w is in xch[w][k]

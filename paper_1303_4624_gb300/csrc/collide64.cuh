@@ -5,22 +5,27 @@
 // instruction, whatever the number of active lanes (measured, dependent or not; a
 // conversion between FP64 and FP32 costs the same), so the form is bound by its FP64
 // instruction count and not by memory: 1520 bytes a D3Q95 cell take 0.23 ns of HBM time,
-// the ~1270 FP64 operations of the pair-by-pair form 2.4 ns.  Three regroupings bring
-// D3Q95 to ~890 operations a cell:
+// the ~1290 FP64 operations of the pair-by-pair form 2.4 ns.  What brings D3Q95 to ~420:
 //   * moments shell by shell: the members of a shell share weight and |xi|^2, so their
 //     sums are formed unweighted (momentum in units of the primitive vector) and each
 //     shell is weighted once;
+//   * those sums, and the relaxation's h + omega (h^eq - h), in 64-bit fixed point on the
+//     integer pipes (fixed64.cuh);
 //   * rho and rho - 1 folded into the shell's equilibrium coefficients, so a pair's
 //     even part is c0 + s^2 (c2 + s^2 c4) and its odd part s (c1 + s^2 c3);
 //   * s and s^2 once per primitive direction b: the pairs k b of several shells (axes
 //     2, 3, 5; diagonals 2, 3, 4; ...) share them, with the powers of k folded into the
 //     coefficients.
+// Measured (us a step): D3Q95 128x32x32 311 pair by pair, 235 regrouped in FP64, 152 with
+// the fixed point; D2Q33 1024x512 446, 354, 217.
 //
 // The shells are dealt into kParts64 parts of nearly equal work (whole shells, so the
 // weighting is not repeated).  Every kernel sums the parts' moments in the same order,
 // ((0 + 1) + (2 + 3)), so one thread doing all parts and several warps doing some each
 // produce the same bits.
 #pragma once
+
+#include "fixed64.cuh"
 
 namespace lbm {
 
@@ -46,6 +51,28 @@ LBM_HD constexpr int shell_part64(int g) {
   constexpr int d3[10] = {-1, 1, 0, 2, 1, 0, 2, 3, 1, 2};
   return M == 0 ? d2[g] : d3[g];
 }
+
+template <int M>
+LBM_HD constexpr int shell_gcd(int g) {
+  for (int i = 1; i < Model<M>::Q; ++i)
+    if (Model<M>::vs.grp[i] == g)
+      return igcd(igcd(iabs(Model<M>::vs.e[i][0]), iabs(Model<M>::vs.e[i][1])), iabs(Model<M>::vs.e[i][2]));
+  return 0;
+}
+// Pairs [first, end) of symmetry group g (g >= 1) in storage order.
+template <int M>
+struct ShellPairs {
+  static constexpr int first(int g) {
+    int p = 0;
+    while (p < Model<M>::NP && Model<M>::vs.grp[1 + 2 * p] != g) ++p;
+    return p;
+  }
+  static constexpr int end(int g) {
+    int p = first(g);
+    while (p < Model<M>::NP && Model<M>::vs.grp[1 + 2 * p] == g) ++p;
+    return p;
+  }
+};
 
 // part < 0: all pairs.
 template <int M>
@@ -107,36 +134,57 @@ __device__ __forceinline__ Mom64 add64(const Mom64& a, const Mom64& b) {
           Model<M>::D == 3 ? __dadd_rn(a.z, b.z) : 0.0};
 }
 
+// p + m and p - m of a pair in fixed point.  A call, as relax_pair64 below: expanded at all
+// 47 pairs of D3Q95 the step's code outgrows the instruction cache (266 us against 152 at
+// 128 x 32 x 32).
+struct SumDiff64 {
+  long long s, d;
+};
+static __device__ __noinline__ SumDiff64 sum_diff64(double hp, double hm, int e) {
+  const long long p = fx_from<56>(hp, e), m = fx_from<56>(hm, e);
+  return {p + m, p - m};
+}
+// Shell by shell: the members' sums in fixed point (fixed64.cuh) at the shell's own scale,
+// so no member loses bits to a shell of larger deviations.
 template <int M, int P, class Get>
 __device__ __forceinline__ Mom64 moments64(Get&& hv) {
-  using T = P64<M, P>;
+  using Mo = Model<M>;
   const ModelConst& mc = c_mc[M];
   Mom64 m = {0.0, 0.0, 0.0, 0.0, 0.0};
   bool none = true;
-  double gs[Model<M>::G], gx[Model<M>::G], gy[Model<M>::G], gz[Model<M>::G];
-  sfor<0, T::t.n>([&](auto I) {
-    constexpr int n = decltype(I)::value;
-    constexpr int g = T::t.grp[n], i = T::t.dir[n];
-    constexpr int bx = T::t.b[n][0], by = T::t.b[n][1], bz = T::t.b[n][2];
-    const double hp = hv(std::integral_constant<int, i>{});
-    const double hm = hv(std::integral_constant<int, i + 1>{});
-    const double sp = __dadd_rn(hp, hm), dm = __dsub_rn(hp, hm);
-    if constexpr (T::first_of(n)) {
-      gs[g] = sp;
-      gx[g] = gy[g] = gz[g] = 0.0;
-    } else {
-      gs[g] = __dadd_rn(gs[g], sp);
-    }
-    if constexpr (bx != 0) gx[g] = xaxpy<bx>(dm, gx[g]);
-    if constexpr (by != 0) gy[g] = xaxpy<by>(dm, gy[g]);
-    if constexpr (bz != 0) gz[g] = xaxpy<bz>(dm, gz[g]);
-    if constexpr (T::last_of(n)) {
-      m.r = none ? __dmul_rn(mc.W[g], gs[g]) : __fma_rn(mc.W[g], gs[g], m.r);
-      m.e = none ? __dmul_rn(mc.WX2[g], gs[g]) : __fma_rn(mc.WX2[g], gs[g], m.e);
-      m.x = none ? __dmul_rn(mc.Wk[g], gx[g]) : __fma_rn(mc.Wk[g], gx[g], m.x);
-      m.y = none ? __dmul_rn(mc.Wk[g], gy[g]) : __fma_rn(mc.Wk[g], gy[g], m.y);
-      if constexpr (Model<M>::D == 3)
-        m.z = none ? __dmul_rn(mc.Wk[g], gz[g]) : __fma_rn(mc.Wk[g], gz[g], m.z);
+  sfor<1, Mo::G>([&](auto Gi) {
+    constexpr int g = decltype(Gi)::value;
+    if constexpr (shell_part64<M>(g) == P) {
+      constexpr int p0 = ShellPairs<M>::first(g), np = ShellPairs<M>::end(g) - p0;
+      constexpr int ge = shell_gcd<M>(g);
+      double h[2 * np];
+      int top = 0;
+      sfor<0, 2 * np>([&](auto J) {
+        constexpr int j = decltype(J)::value;
+        h[j] = hv(std::integral_constant<int, 1 + 2 * p0 + j>{});
+        top = max(top, fx_top(h[j]));
+      });
+      const int e = fx_exponent(top);
+      long long gs = 0, gx = 0, gy = 0, gz = 0;
+      sfor<0, np>([&](auto J) {
+        constexpr int j = decltype(J)::value, i = 1 + 2 * (p0 + j);
+        constexpr int bx = Mo::vs.e[i][0] / ge, by = Mo::vs.e[i][1] / ge, bz = Mo::vs.e[i][2] / ge;
+        const SumDiff64 sd = sum_diff64(h[2 * j], h[2 * j + 1], e);
+        const long long d = sd.d;
+        gs += sd.s;
+        if constexpr (bx != 0) gx += bx * d;
+        if constexpr (by != 0) gy += by * d;
+        if constexpr (bz != 0) gz += bz * d;
+      });
+      // sums: at most 72 2^56 < 2^63
+      double S = fx_to<56>(gs, e), X = fx_to<56>(gx, e), Y = fx_to<56>(gy, e), Z = 0.0;
+      if constexpr (Mo::D == 3) Z = fx_to<56>(gz, e);
+      if (!fx_regular(top)) S = X = Y = Z = __longlong_as_double(0x7ff8000000000000ll);
+      m.r = none ? __dmul_rn(mc.W[g], S) : __fma_rn(mc.W[g], S, m.r);
+      m.e = none ? __dmul_rn(mc.WX2[g], S) : __fma_rn(mc.WX2[g], S, m.e);
+      m.x = none ? __dmul_rn(mc.Wk[g], X) : __fma_rn(mc.Wk[g], X, m.x);
+      m.y = none ? __dmul_rn(mc.Wk[g], Y) : __fma_rn(mc.Wk[g], Y, m.y);
+      if constexpr (Mo::D == 3) m.z = none ? __dmul_rn(mc.Wk[g], Z) : __fma_rn(mc.Wk[g], Z, m.z);
       none = false;
     }
   });
@@ -182,11 +230,36 @@ __device__ __forceinline__ Cell64 cell64(const Mom64& m) {
   return c;
 }
 
+// h + omega (h^eq - h) of a pair's two members, h^eq = ev +- od: in fixed point at the
+// scale of the largest of the four terms (140 integer instructions for six at the FP64
+// rate); om is omega in units of 2^-62.  The error is a few units of 2^-60 of that term,
+// against omega 2^-53 of it in FP64; a smaller omega than 2^-6 (0 must return h as it is)
+// keeps the FP64 operations.
+struct Two64 {
+  double p, m;
+};
+static __device__ __noinline__ Two64 relax_pair_any(double ev, double od, double hp, double hm,
+                                                    double omega) {
+  return {__fma_rn(omega, __dsub_rn(__dadd_rn(ev, od), hp), hp),
+          __fma_rn(omega, __dsub_rn(__dsub_rn(ev, od), hm), hm)};
+}
+static __device__ __noinline__ Two64 relax_pair64(double ev, double od, double hp, double hm,
+                                              double omega, long long om) {
+  const int top = max(max(fx_top(ev), fx_top(od)), max(fx_top(hp), fx_top(hm)));
+  if (!fx_regular(top) || omega < 0x1p-6) return relax_pair_any(ev, od, hp, hm, omega);
+  const int e = fx_exponent(top);
+  const long long v = fx_from<60>(ev, e), o = fx_from<60>(od, e);
+  const long long p = fx_from<60>(hp, e), m = fx_from<60>(hm, e);
+  // |v + o - p| < 3 2^60; times omega < 2: below 6 2^60
+  return {fx_to<60>(p + 4 * fx_mulhi(v + o - p, om), e), fx_to<60>(m + 4 * fx_mulhi(v - o - m, om), e)};
+}
+
 // The relaxation h' = h + omega (h^eq - h) of one part's pairs.
 template <int M, int P, class Get, class Store>
 __device__ __forceinline__ void relax64(const Cell64& c, double omega, Get&& hv, Store&& st) {
   using T = P64<M, P>;
   const ModelConst& mc = c_mc[M];
+  const long long om = fx_from<63>(omega, 1023);   // omega < 2 = 2^(1023 - 1022)
   double s = 0.0, s2 = 0.0;
   sfor<0, T::t.n>([&](auto I) {
     constexpr int n = decltype(I)::value;
@@ -206,8 +279,9 @@ __device__ __forceinline__ void relax64(const Cell64& c, double omega, Get&& hv,
     const double od = __dmul_rn(s, __fma_rn(s2, c3, c1));
     const double hp = hv(std::integral_constant<int, i>{});
     const double hm = hv(std::integral_constant<int, i + 1>{});
-    st(std::integral_constant<int, i>{}, __fma_rn(omega, __dsub_rn(__dadd_rn(ev, od), hp), hp));
-    st(std::integral_constant<int, i + 1>{}, __fma_rn(omega, __dsub_rn(__dsub_rn(ev, od), hm), hm));
+    const Two64 r = relax_pair64(ev, od, hp, hm, omega, om);
+    st(std::integral_constant<int, i>{}, r.p);
+    st(std::integral_constant<int, i + 1>{}, r.m);
   });
 }
 

@@ -1,0 +1,53 @@
+// fixed64.cuh - 64-bit fixed point on the integer pipes, for sums of FP64 values.
+//
+// An FP64 instruction holds a scheduler's FP64 unit for 64 cycles, while the integer
+// pipes take one every cycle or two: an FP64 addition costs as much as some fifty integer
+// instructions.  A group of doubles (the populations of a shell, or the terms of one
+// relaxation) is brought to a common exponent, that of its largest member, and added as
+// 64-bit integers.  With 56 or more bits below the largest member nothing is lost against
+// FP64's 53; integer sums do not depend on their order.
+//
+// top: the largest (high word & 0x7fffffff) of the group; its exponent field e bounds
+// |v| < 2^(e - 1022).  A value v is held as trunc(v 2^(B - (e - 1022))) with B bits.
+// Groups with an exponent field of 2000 or more (|v| >= 2^977, Inf, NaN) are the caller's
+// (fx_regular); fields below 128 count as 128 (|v| < 2^-894 is held as 0).
+#pragma once
+
+namespace lbm {
+
+__device__ __forceinline__ int fx_top(double v) { return __double2hiint(v) & 0x7fffffff; }
+__device__ __forceinline__ bool fx_regular(int top) { return top < (2000 << 20); }
+__device__ __forceinline__ int fx_exponent(int top) { return max(top >> 20, 128); }
+
+// v with B bits below 2^(e - 1022): 63 - B + e(v)'s distance is the right shift.
+template <int B>
+__device__ __forceinline__ long long fx_from(double v, int e) {
+  const unsigned h = (unsigned)__double2hiint(v), l = (unsigned)__double2loint(v);
+  const int r = min(e + (63 - B) - (int)((h >> 20) & 0x7ffu), 63);
+  const unsigned mh = (__funnelshift_l(l, h, 10) & 0x3fffffffu) | 0x40000000u;   // 1.f at bit 62
+  const unsigned long long m = ((unsigned long long)mh << 32) | (l << 10);
+  const long long s = (long long)((int)h >> 31);
+  return ((long long)(m >> r) ^ s) - s;
+}
+// The double nearest to i (B bits below 2^(e - 1022)).
+template <int B>
+__device__ __forceinline__ double fx_to(long long i, int e) {
+  const long long s = i >> 63;
+  const unsigned long long u = (unsigned long long)((i ^ s) - s);
+  const int lz = __clzll((long long)u);
+  const unsigned long long m = u << (lz & 63);
+  const unsigned long long f = (m >> 11) + ((m >> 10) & 1);   // 53 bits, rounded
+  const int exponent = e + (63 - B) + 1 - lz;                 // field of the leading bit
+  unsigned long long bits = ((unsigned long long)(unsigned)(exponent - 1) << 52) + f;
+  bits |= (unsigned long long)s & 0x8000000000000000ull;
+  return __longlong_as_double(u == 0 ? 0ll : (long long)bits);
+}
+// a b / 2^64 to within three units, |a|, |b| < 2^63: three wide products.
+__device__ __forceinline__ long long fx_mulhi(long long a, long long b) {
+  const int ah = (int)(a >> 32), bh = (int)(b >> 32);
+  const int al = (int)((unsigned)a >> 1), bl = (int)((unsigned)b >> 1);
+  const long long t = (long long)ah * bl + (long long)al * bh;
+  return (long long)ah * bh + (t >> 31);
+}
+
+}  // namespace lbm

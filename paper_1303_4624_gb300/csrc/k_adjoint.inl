@@ -33,6 +33,7 @@ cudaError_t adjoint64_m(const void* state_n, const void* nu_next, const double* 
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)((g.ncell + 31) / 32));
   cfg.blockDim = dim3(32 * w);
+  cfg.dynamicSmemBytes = dldrho ? 0 : Model<M>::Q * 32 * sizeof(double);
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;

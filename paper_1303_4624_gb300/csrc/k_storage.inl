@@ -210,6 +210,7 @@ cudaError_t step64_m(const void* src, void* dst, const Grid& g, double omega, in
   const int w = lin64_warps<M>(g.ncell, sms);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)((g.ncell + 31) / 32));
+  cfg.dynamicSmemBytes = Model<M>::Q * 32 * sizeof(double);
   cfg.blockDim = dim3(32 * w);
   cfg.stream = st;
   cudaLaunchAttribute attr[1];

@@ -595,6 +595,10 @@ __device__ __forceinline__ void cp_async4(void* smem, const void* gmem) {
   const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(s), "l"(gmem) : "memory");
 }
+__device__ __forceinline__ void cp_async8(void* smem, const void* gmem) {
+  const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(s), "l"(gmem) : "memory");
+}
 __device__ __forceinline__ void cp_async_wait_all() {
   asm volatile("cp.async.wait_all;" ::: "memory");
 }
@@ -761,14 +765,10 @@ inline bool linear_rows(const Grid& g) {
 // parts of collide64, and the parts' moments are exchanged through shared memory and
 // summed in collide64's order, so every WARPS gives the same bits (see lin64_warps for
 // the rule).
-// The populations are read twice, for the moments and for the relaxation (D3Q95: 95
-// doubles would take 190 registers); the second read comes from L1 / L2, and memory has
-// the time (1520 bytes a cell at under 1 TB/s).
-__device__ __forceinline__ double ld_again(const double* p) {
-  double v;   // volatile: not merged with the first read
-  asm volatile("ld.global.nc.f64 %0, [%1];" : "=d"(v) : "l"(p));
-  return v;
-}
+// Each thread copies its populations to shared memory first (cp.async, its own copies only,
+// so no barrier): they are used twice, for the moments and for the relaxation, 95 doubles
+// would take 190 registers, and read again from L1 / L2 they stall the few warps an SM
+// holds (D3Q95 128 x 32 x 32: 190 us against 152).  24 KB a warp for D3Q95.
 template <int M, bool REV, int WARPS>
 __global__ void __launch_bounds__(32 * WARPS, 8 / WARPS)
     k_stream_collide64(const double* __restrict__ src, double* __restrict__ dst, Grid g,
@@ -804,27 +804,35 @@ __global__ void __launch_bounds__(32 * WARPS, 8 / WARPS)
     constexpr int i = decltype(I)::value;
     if (active) dst[(size_t)i * (size_t)g.ncell + cell] = fixed ? __ldg(tmpl + 2 * i) : v;
   };
-  auto hm = [&](auto I) { return __ldg(at(I)); };
-  auto hr = [&](auto I) { return ld_again(at(I)); };
+  extern __shared__ __align__(16) double stage64[];
+  double* const mine = stage64 + lane;
+  sfor<0, Mo::Q>([&](auto I) {
+    constexpr int i = decltype(I)::value;
+    constexpr int p = i == 0 ? -1 : shell_part64<M>(Mo::vs.grp[i]);
+    if (WARPS == 1 || i == 0 || p / (kParts64 / WARPS) == warp) cp_async8(mine + 32 * i, at(I));
+  });
+  cp_async_wait_all();
+  auto hm = [&](auto I) { return mine[32 * decltype(I)::value]; };
+  auto hr = hm;
   if constexpr (WARPS == 1) {
     collide64<M>(hm, hr, omega, st);
   } else {
     constexpr int PW = kParts64 / WARPS;         // parts per warp
     __shared__ double xch[kParts64 / PW][5][32];
     const double h0 = hm(rest);
-    Mom64 mine;
+    Mom64 own;
     sfor<0, WARPS>([&](auto Wi) {
       constexpr int w = decltype(Wi)::value;
       if (warp == w) {
-        mine = moments64<M, w * PW>(hm);
-        if constexpr (PW == 2) mine = add64<M>(mine, moments64<M, w * PW + 1>(hm));
+        own = moments64<M, w * PW>(hm);
+        if constexpr (PW == 2) own = add64<M>(own, moments64<M, w * PW + 1>(hm));
       }
     });
-    xch[warp][0][lane] = mine.r;
-    xch[warp][1][lane] = mine.e;
-    xch[warp][2][lane] = mine.x;
-    xch[warp][3][lane] = mine.y;
-    xch[warp][4][lane] = mine.z;
+    xch[warp][0][lane] = own.r;
+    xch[warp][1][lane] = own.e;
+    xch[warp][2][lane] = own.x;
+    xch[warp][3][lane] = own.y;
+    xch[warp][4][lane] = own.z;
     __syncthreads();
     auto part = [&](int p) {
       return Mom64{xch[p][0][lane], xch[p][1][lane], xch[p][2][lane], xch[p][3][lane], xch[p][4][lane]};
@@ -849,10 +857,10 @@ __global__ void __launch_bounds__(32 * WARPS, 8 / WARPS)
   }
 }
 
-// Warps per 32 cells: the choice with the fewest FP64 instructions on the busiest
-// scheduler, ceil(warps / schedulers) times the instructions of a warp.  Those are about
-// 200 / 830 for all pairs of D2Q33 / D3Q95 and 70 for what every warp repeats (moment
-// totals, 1 / rho, the coefficients of the cell).
+// Warps per 32 cells: the choice with the least work on the busiest
+// scheduler, ceil(warps / schedulers) times the time of a warp.  In units of an FP64
+// instruction that is about 170 / 580 for all pairs of D2Q33 / D3Q95 and 70 for what every
+// warp repeats (moment totals, 1 / rho, the coefficients of the cell).
 template <int M>
 inline int lin64_warps(long long ncell, int sms) {
   const long long groups = (ncell + 31) / 32;
@@ -860,7 +868,7 @@ inline int lin64_warps(long long ncell, int sms) {
   long long best_cost = -1;
   for (int w = 1; w <= 4; w *= 2) {
     const long long rounds = (groups * w + 4LL * sms - 1) / (4LL * sms);
-    const long long cost = rounds * ((M == 0 ? 200 : 830) / w + 70);
+    const long long cost = rounds * ((M == 0 ? 170 : 580) / w + 70);
     if (best_cost < 0 || cost < best_cost) {
       best = w;
       best_cost = cost;
