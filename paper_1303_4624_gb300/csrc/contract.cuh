@@ -20,15 +20,15 @@
 
 namespace lbm {
 
-// Arithmetic of the two number types.
+// Arithmetic of the two number types (double-float not renormalised between operations).
 __device__ __forceinline__ double nadd(double a, double b) { return __dadd_rn(a, b); }
 __device__ __forceinline__ double nsub(double a, double b) { return __dsub_rn(a, b); }
 __device__ __forceinline__ double nmul(double a, double b) { return __dmul_rn(a, b); }
 __device__ __forceinline__ double nfma(double a, double b, double c) { return __fma_rn(a, b, c); }
-__device__ __forceinline__ FF nadd(FF a, FF b) { return ff_add(a, b); }
-__device__ __forceinline__ FF nsub(FF a, FF b) { return ff_add(a, ff_neg(b)); }
-__device__ __forceinline__ FF nmul(FF a, FF b) { return ff_mul(a, b); }
-__device__ __forceinline__ FF nfma(FF a, FF b, FF c) { return ff_add(ff_mul(a, b), c); }
+__device__ __forceinline__ FF nadd(FF a, FF b) { return fu_add(a, b); }
+__device__ __forceinline__ FF nsub(FF a, FF b) { return fu_add(a, ff_neg(b)); }
+__device__ __forceinline__ FF nmul(FF a, FF b) { return fu_mul(a, b); }
+__device__ __forceinline__ FF nfma(FF a, FF b, FF c) { return fu_add(c, fu_mul(a, b)); }
 // A compile-time constant; its double-float form is the exact split.
 template <class R>
 __device__ __forceinline__ R ncst(double v) {
@@ -43,12 +43,12 @@ __device__ __forceinline__ R ncst(double v) {
 template <int K, class R>
 __device__ __forceinline__ R nscale(R v) {
   if constexpr (K == 1) return v;
-  else if constexpr (std::is_same<R, FF>::value) return ff_scale<K>(v);
+  else if constexpr (std::is_same<R, FF>::value) return fu_scale<K>(v);
   else return K == -1 ? -v : __dmul_rn((double)K, v);
 }
 template <int K, class R>
 __device__ __forceinline__ R naxpy(R v, R acc) {
-  if constexpr (std::is_same<R, FF>::value) return ff_add(ff_scale<K>(v), acc);
+  if constexpr (std::is_same<R, FF>::value) return fu_add(acc, fu_scale<K>(v));
   else return xaxpy<K>(v, acc);
 }
 template <int EX, int EY, int EZ, class R>

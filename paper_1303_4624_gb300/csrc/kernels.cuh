@@ -746,11 +746,11 @@ __global__ void __launch_bounds__(kLinThreads, DirectMinBlocks<M, S>::value * 12
 // 22.3 / 22.6.
 template <int M, class S>
 inline bool linear_rows(const Grid& g) {
-#ifdef LBM_LIN_ALWAYS
-  return LBM_LIN_ALWAYS;
-#endif
   const int bx = cell_block_x(g.nx);
   const long long padded = (long long)(g.nx + bx - 1) / bx * bx;
+  // The 16-bit forms are bound by issue and pay more for the lanes' own offsets (D3Q95 FP16
+  // 250x67x21 32.2 / 40.8, 201x99x50 with 21 % idle 104 / 116, 33x33x33 with 48 % 7.5 / 7.0).
+  if (sizeof(S) == 2) return padded * 10 > (long long)g.nx * 14;
   if (padded * 16 > (long long)g.nx * 17) return true;
   return g.nx * sizeof(S) % 32 != 0 &&
          (size_t)Model<M>::Q * (size_t)g.ncell * sizeof(S) > ((size_t)128 << 20);
@@ -970,6 +970,22 @@ __device__ __forceinline__ FF ff_from(double d) {
   const float hi = __double2float_rn(d);
   return {hi, __double2float_rn(d - (double)hi)};
 }
+// d as a double-float pair without the conversion instruction: hi its leading 24 bits
+// (truncated), lo the other 29 rounded to 24.  False (nothing set) outside 2^-63 <= |d| < 2^64.
+__device__ __forceinline__ bool ff_split(double d, FF* v) {
+  const unsigned h = (unsigned)__double2hiint(d), l = (unsigned)__double2loint(d);
+  const unsigned m = h & 0x7fffffffu, e = m >> 20, sign = h & 0x80000000u;
+  if ((m | l) == 0) {
+    *v = {__uint_as_float(sign), 0.f};
+    return true;
+  }
+  if (e < 960u || e >= 1087u) return false;
+  v->hi = __uint_as_float(sign | __funnelshift_l(l, m - 0x38000000u, 3));
+  const float scale = __uint_as_float(sign | ((e - 948u) << 23));   // 2^(e - 1023 - 52)
+  v->lo = __fmul_rn((float)(l & 0x1fffffffu), scale);
+  return true;
+}
+
 __device__ __forceinline__ FF ff_renorm(float p, float e) {
   const float h = __fadd_rn(p, e);
   return {h, __fsub_rn(e, __fsub_rn(h, p))};
@@ -997,6 +1013,26 @@ __device__ __forceinline__ FF ff_scale(FF a) {
 __device__ __forceinline__ FF ff_neg(FF a) { return {-a.hi, -a.lo}; }
 __device__ __forceinline__ FF ff_const(float c) { return {c, 0.f}; }
 
+// Without the final renormalisation: hi + lo is exact to ~2^-46 of the result, lo up to a
+// few ulps of hi.  Enough between the steps of a polynomial.
+__device__ __forceinline__ FF fu_mul(FF a, FF b) {
+  const float p = __fmul_rn(a.hi, b.hi);
+  float e = __fmaf_rn(a.hi, b.hi, -p);
+  e = __fmaf_rn(a.hi, b.lo, e);
+  return {p, __fmaf_rn(a.lo, b.hi, e)};
+}
+__device__ __forceinline__ FF fu_add(FF a, FF b) {
+  float s, e;
+  two_sum(a.hi, b.hi, s, e);
+  return {s, __fadd_rn(e, __fadd_rn(a.lo, b.lo))};
+}
+template <int K>
+__device__ __forceinline__ FF fu_scale(FF a) {
+  if constexpr ((K & (K - 1)) == 0) return {(float)K * a.hi, (float)K * a.lo};   // exact
+  const float p = __fmul_rn((float)K, a.hi);
+  return {p, __fmaf_rn((float)K, a.lo, __fmaf_rn((float)K, a.hi, -p))};
+}
+
 // hi + lo rounded once to the storage type.  FP32: one add.  FP16 / BF16: round hi,
 // unless hi is exactly halfway between two neighbours of the 16-bit format (FP32
 // holds those midpoints exactly), where the sign of lo decides; since hi is hi + lo
@@ -1008,21 +1044,38 @@ template <>
 __device__ __forceinline__ float ff_round<float>(FF v) {
   return __fadd_rn(v.hi, v.lo);
 }
-template <>
-__device__ __forceinline__ __half ff_round<__half>(FF v) {
+// The midpoint test on hi's bits: the 13 (16) dropped bits are 1000...  That is the test for
+// normal FP16 results; subnormal ones (|hi| < 2^-14) compare hi with the two neighbours'
+// mean, in a call (expanded, its conversions are predicated into every result).
+static __device__ __noinline__ __half ff_round_half_any(FF v) {
   const __half a = __float2half_rd(v.hi), b = __float2half_ru(v.hi);
   if (v.lo != 0.f && __half_as_ushort(a) != __half_as_ushort(b) &&
       v.hi == 0.5f * (__half2float(a) + __half2float(b)))
     return v.lo > 0.f ? b : a;
   return __float2half_rn(v.hi);
 }
-template <>
-__device__ __forceinline__ __nv_bfloat16 ff_round<__nv_bfloat16>(FF v) {
+static __device__ __noinline__ __nv_bfloat16 ff_round_bf16_any(FF v) {
   const __nv_bfloat16 a = __float2bfloat16_rd(v.hi), b = __float2bfloat16_ru(v.hi);
   if (v.lo != 0.f && __bfloat16_as_ushort(a) != __bfloat16_as_ushort(b) &&
       v.hi == 0.5f * (__bfloat162float(a) + __bfloat162float(b)))
     return v.lo > 0.f ? b : a;
   return __float2bfloat16_rn(v.hi);
+}
+template <>
+__device__ __forceinline__ __half ff_round<__half>(FF v) {
+  const unsigned u = __float_as_uint(v.hi);
+  if ((u & 0x1fffu) == 0x1000u || (u & 0x7fffffffu) < 0x38800000u) return ff_round_half_any(v);
+  return __float2half_rn(v.hi);
+}
+template <>
+__device__ __forceinline__ __nv_bfloat16 ff_round<__nv_bfloat16>(FF v) {
+  if ((__float_as_uint(v.hi) & 0xffffu) == 0x8000u) return ff_round_bf16_any(v);
+  return __float2bfloat16_rn(v.hi);
+}
+// ff_round of the 16-bit types wants hi = hi + lo rounded to FP32; of FP32 it adds them.
+template <class S>
+__device__ __forceinline__ FF ff_out(FF v) {
+  if constexpr (sizeof(S) == 4) return v; else return ff_renorm(v.hi, v.lo);
 }
 
 // s = e . (a u) as double-float for a compile-time lattice vector e
@@ -1074,33 +1127,72 @@ __global__ void __launch_bounds__(256)
     const FF rm1 = ff_add(r, ff_const(-1.f));
     const FF vx = ff_mul(ux, a), vy = ff_mul(uy, a), vz = ff_mul(uz, a);
     const FF r6 = ff_mul(r, FF{c6h, c6l}), r24 = ff_mul(r, FF{c24h, c24l});
-    {
-      const FF h0 = ff_add(rm1, ff_mul(r, K0m1));
-      dst[idx] = ff_round<S>(h0);   // one rounding to the storage type
-    }
-    FF R0 = {0.f, 0.f}, R1 = R0, R2 = R0;
-    sfor<0, NP>([&](auto P) {
-      constexpr int p = decltype(P)::value;
-      constexpr int ip = 1 + 2 * p, im = 2 + 2 * p;
-      constexpr int gg = Mo::vs.grp[ip];
-      constexpr bool first = (p == 0) || (Mo::vs.grp[ip - 2] != gg);
-      constexpr int ex = Mo::vs.e[ip][0], ey = Mo::vs.e[ip][1], ez = Mo::vs.e[ip][2];
-      if constexpr (first) {   // the shell's coefficients, once per shell
-        const FF x2 = {mc.X2f[gg], mc.X2lo[gg]};
-        const FF A0m1 = ff_add(K0m1, ff_mul(x2, ff_add(K1, ff_mul(x2, K2))));
-        R0 = ff_add(rm1, ff_mul(r, A0m1));
-        R1 = ff_mul(r, ff_add(L0, ff_mul(L1, x2)));
-        R2 = ff_mul(r, ff_add(M0, ff_mul(M1, x2)));
+    if constexpr (sizeof(S) == 2) {
+      // 16-bit forms: the pairs of a primitive direction share s and s^2, rho is folded into
+      // the shells' coefficients and the sums are not renormalised in between: 5000
+      // instructions a D3Q95 cell against 6800 (8.2 -> 6.4 ms for 512 x 256 x 256, bound by
+      // issue), with ~46 significant bits before the one rounding.  The FP32 form, where that
+      // would round about one result in 2^20 the other way, keeps the renormalised sums.
+      // EqCoef's coefficients times rho
+      const FF P0 = ff_add(rm1, ff_mul(r, K0m1)), rK1 = ff_mul(r, K1), rK2 = ff_mul(r, K2);
+      const FF rL0 = ff_mul(r, L0), rL1 = ff_mul(r, L1), rM0 = ff_mul(r, M0), rM1 = ff_mul(r, M1);
+      // Per shell R0, k R1, k^2 R2, k^3 rho / 6, k^4 rho / 24 (its pairs are +- k b), formed at
+      // the shell's first pair; s = b . v and s^2 once per primitive direction b.  The pairs
+      // go direction by direction (P64<M, -1>).
+      dst[idx] = ff_round<S>(P0);       // one rounding to the storage type
+      using T = P64<M, -1>;
+      FF R0[Mo::G], R1[Mo::G], R2[Mo::G], R3[Mo::G], R4[Mo::G];   // indexed at compile time
+      FF s = {0.f, 0.f}, s2 = s;
+      sfor<0, NP>([&](auto P) {
+        constexpr int n = decltype(P)::value;
+        constexpr int gg = T::t.grp[n], k = T::t.k[n], ip = T::t.dir[n], im = ip + 1;
+        constexpr int bx = T::t.b[n][0], by = T::t.b[n][1], bz = T::t.b[n][2];
+        if constexpr (T::first_of(n)) {
+          const FF x2 = {mc.X2f[gg], mc.X2lo[gg]};
+          R0[gg] = fu_add(P0, fu_mul(x2, fu_add(rK1, fu_mul(x2, rK2))));
+          R1[gg] = fu_scale<k>(fu_add(rL0, fu_mul(rL1, x2)));
+          R2[gg] = fu_scale<k * k>(fu_add(rM0, fu_mul(rM1, x2)));
+          R3[gg] = fu_scale<k * k * k>(r6);
+          R4[gg] = fu_scale<k * k * k * k>(r24);
+        }
+        if constexpr (T::new_base(n)) {
+          s = ff_edot<bx, by, bz>(vx, vy, vz);
+          s2 = fu_mul(s, s);
+        }
+        const FF ev = fu_add(R0[gg], fu_mul(s2, fu_add(R2[gg], fu_mul(s2, R4[gg]))));
+        const FF od = fu_mul(s, fu_add(R1[gg], fu_mul(s2, R3[gg])));
+        dst[(size_t)ip * g.ncell + idx] = ff_round<S>(ff_out<S>(fu_add(ev, od)));
+        dst[(size_t)im * g.ncell + idx] = ff_round<S>(ff_out<S>(fu_add(ev, ff_neg(od))));
+      });
+    } else {
+      {
+        const FF h0 = ff_add(rm1, ff_mul(r, K0m1));
+        dst[idx] = ff_round<S>(h0);   // one rounding to the storage type
       }
-      const FF s = ff_edot<ex, ey, ez>(vx, vy, vz);
-      const FF s2 = ff_mul(s, s);
-      const FF ev = ff_add(R0, ff_mul(s2, ff_add(R2, ff_mul(s2, r24))));
-      const FF od = ff_mul(s, ff_add(R1, ff_mul(s2, r6)));
-      const FF hp = ff_add(ev, od);
-      const FF hm = ff_add(ev, ff_neg(od));
-      dst[(size_t)ip * g.ncell + idx] = ff_round<S>(hp);
-      dst[(size_t)im * g.ncell + idx] = ff_round<S>(hm);
-    });
+      FF R0 = {0.f, 0.f}, R1 = R0, R2 = R0;
+      sfor<0, NP>([&](auto P) {
+        constexpr int p = decltype(P)::value;
+        constexpr int ip = 1 + 2 * p, im = 2 + 2 * p;
+        constexpr int gg = Mo::vs.grp[ip];
+        constexpr bool first = (p == 0) || (Mo::vs.grp[ip - 2] != gg);
+        constexpr int ex = Mo::vs.e[ip][0], ey = Mo::vs.e[ip][1], ez = Mo::vs.e[ip][2];
+        if constexpr (first) {   // the shell's coefficients, once per shell
+          const FF x2 = {mc.X2f[gg], mc.X2lo[gg]};
+          const FF A0m1 = ff_add(K0m1, ff_mul(x2, ff_add(K1, ff_mul(x2, K2))));
+          R0 = ff_add(rm1, ff_mul(r, A0m1));
+          R1 = ff_mul(r, ff_add(L0, ff_mul(L1, x2)));
+          R2 = ff_mul(r, ff_add(M0, ff_mul(M1, x2)));
+        }
+        const FF s = ff_edot<ex, ey, ez>(vx, vy, vz);
+        const FF s2 = ff_mul(s, s);
+        const FF ev = ff_add(R0, ff_mul(s2, ff_add(R2, ff_mul(s2, r24))));
+        const FF od = ff_mul(s, ff_add(R1, ff_mul(s2, r6)));
+        const FF hp = ff_add(ev, od);
+        const FF hm = ff_add(ev, ff_neg(od));
+        dst[(size_t)ip * g.ncell + idx] = ff_round<S>(hp);
+        dst[(size_t)im * g.ncell + idx] = ff_round<S>(hm);
+      });
+    }
     return;
   }
   const double r = rho[idx];
@@ -1423,22 +1515,6 @@ __device__ __forceinline__ double widen(float v) {
   const unsigned hi = (u & 0x80000000u) | (zero ? 0u : (m >> 3) + 0x38000000u);
   return __hiloint2double((int)hi, (int)(u << 29));
 }
-// d as a double-float pair without the conversion instruction: hi its leading 24 bits
-// (truncated), lo the other 29 rounded to 24.  False (nothing set) outside 2^-63 <= |d| < 2^64.
-__device__ __forceinline__ bool ff_split(double d, FF* v) {
-  const unsigned h = (unsigned)__double2hiint(d), l = (unsigned)__double2loint(d);
-  const unsigned m = h & 0x7fffffffu, e = m >> 20, sign = h & 0x80000000u;
-  if ((m | l) == 0) {
-    *v = {__uint_as_float(sign), 0.f};
-    return true;
-  }
-  if (e < 960u || e >= 1087u) return false;
-  v->hi = __uint_as_float(sign | __funnelshift_l(l, m - 0x38000000u, 3));
-  const float scale = __uint_as_float(sign | ((e - 948u) << 23));   // 2^(e - 1023 - 52)
-  v->lo = __fmul_rn((float)(l & 0x1fffffffu), scale);
-  return true;
-}
-
 // The weight of flat element k's direction, kept in registers until an element of another
 // direction comes.
 struct IoWeight {
