@@ -254,7 +254,10 @@ cudaError_t step_m(const void* src, void* dst, const Grid& g, double omega, int 
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    if (ends.width > 0 || linear_rows<M, S>(g)) {
+    int sms = 0;
+    cudaError_t e = sm_count(&sms);
+    if (e != cudaSuccess) return e;
+    if (ends.width > 0 || linear_rows<M, S>(g, sms)) {
       cfg.gridDim = dim3((unsigned)((g.ncell + kLinThreads - 1) / kLinThreads));
       cfg.blockDim = dim3(kLinThreads);
       return cudaLaunchKernelEx(&cfg, linear_kernel<M>(g, rev, ends.width > 0),

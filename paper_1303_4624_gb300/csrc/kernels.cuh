@@ -692,10 +692,7 @@ __global__ void __launch_bounds__(128, DirectMinBlocks<M, S>::value)
 // ENDS: the fixed end planes are written here as well (a cell of an end plane stores its
 // template and gathers nothing) instead of by a second kernel after the step.
 // In y and z only the offsets that occur are formed; lanes of a warp differ in them.
-#ifndef LBM_LIN_THREADS
-#define LBM_LIN_THREADS 128
-#endif
-constexpr int kLinThreads = LBM_LIN_THREADS;
+constexpr int kLinThreads = 128;   // 64 and 32 measured slower (512x256x256 3902, 4029, 4136 us)
 template <int M, class S, bool REV, bool NARROW, bool ENDS>
 __global__ void __launch_bounds__(kLinThreads, DirectMinBlocks<M, S>::value * 128 / kLinThreads)
     k_stream_collide_linear(const S* __restrict__ src, S* __restrict__ dst, Grid g, double omega,
@@ -744,13 +741,18 @@ __global__ void __launch_bounds__(kLinThreads, DirectMinBlocks<M, S>::value * 12
 // start off the 32-byte sectors cost partial sector writes once the state leaves L2:
 // 250x64x64 131 / 125, D2Q33 2046x1024 90.1 / 82.7, but D2Q33 1021x515 (two copies of 69 MB)
 // 22.3 / 22.6.
+// A grid of at most one wave of warps is latency-bound, and the linear kernel's divisions
+// lengthen its chain (56x30x30 8.3 / 8.9, 48x20x20 5.3 / 5.5, D2Q33 72x300 2.6 / 2.9): there
+// the line is at three idle lanes in seven (33x33x33 8.2 / 6.4, 16x14x24 5.2 / 4.4).
 template <int M, class S>
-inline bool linear_rows(const Grid& g) {
+inline bool linear_rows(const Grid& g, int sms) {
   const int bx = cell_block_x(g.nx);
   const long long padded = (long long)(g.nx + bx - 1) / bx * bx;
   // The 16-bit forms are bound by issue and pay more for the lanes' own offsets (D3Q95 FP16
   // 250x67x21 32.2 / 40.8, 201x99x50 with 21 % idle 104 / 116, 33x33x33 with 48 % 7.5 / 7.0).
   if (sizeof(S) == 2) return padded * 10 > (long long)g.nx * 14;
+  const long long wave = (long long)sms * DirectMinBlocks<M, S>::value * 128;
+  if (padded * g.ny * g.nz <= wave) return padded * 4 > (long long)g.nx * 7;
   if (padded * 16 > (long long)g.nx * 17) return true;
   return g.nx * sizeof(S) % 32 != 0 &&
          (size_t)Model<M>::Q * (size_t)g.ncell * sizeof(S) > ((size_t)128 << 20);
