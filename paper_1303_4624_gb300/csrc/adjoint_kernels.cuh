@@ -42,13 +42,6 @@ struct EqGrad {
 };
 
 
-// Passes 2 and 3 as loops over each shell's pairs (lattice vectors read from
-// constant memory) instead of fully unrolled over all pairs: a smaller kernel for
-// the instruction cache.  Needs lambda in shared memory or uniform (FP32 adjoint).
-#ifndef LBM_ADJ_SHELL_LOOP
-#define LBM_ADJ_SHELL_LOOP 1
-#endif
-
 __device__ __forceinline__ double block_sum_128(double v, double* sh) {
   v = warp_sum(v);
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -76,25 +69,13 @@ constexpr int kAdjUnroll = LBM_ADJ_UNROLL;
 #ifndef LBM_ADJ_GROUPS
 #define LBM_ADJ_GROUPS 4
 #endif
-#ifndef LBM_ADJ_LAM_SMEM
-#define LBM_ADJ_LAM_SMEM 1
-#endif
-template <class S>
-struct AdjMinBlocks {
-  static constexpr int value = std::is_same<S, double>::value ? 1 : LBM_ADJ_MINB;
-};
-// FP32 adjoint: the Q gathered lambda_i of a thread live in dynamic shared memory
-// (lambda_i of thread t at word i * 128 + t: conflict-free), which leaves the
-// registers to the gather offsets and the sums (Q floats in registers on top of
-// them spill at 128 registers a thread).  The FP64 adjoint keeps them in registers.
-template <class L>
-struct AdjLamSmem {
-  static constexpr bool value = std::is_same<L, float>::value && LBM_ADJ_LAM_SMEM;
-};
+// The Q gathered lambda_i of a thread live in dynamic shared memory (lambda_i of thread t at
+// word i * 128 + t: conflict-free), which leaves the registers to the gather offsets and the
+// sums (Q floats in registers on top of them spill at 128 registers a thread).
 constexpr int kAdjThreads = 128;
 template <int M, class L>
 constexpr int adj_smem_bytes() {
-  return AdjLamSmem<L>::value ? Model<M>::Q * kAdjThreads * (int)sizeof(L) : 0;
+  return Model<M>::Q * kAdjThreads * (int)sizeof(L);
 }
 // Address of population i at a cell: the element index in 32 bits when every index
 // of a state copy fits them (NARROW), which saves the per-population 64-bit offset
@@ -105,14 +86,13 @@ constexpr int adj_smem_bytes() {
   (NARROW ? (base) + (uint32_t)((uint32_t)(i) * (uint32_t)g.ncell + (uint32_t)(cell))         \
           : (base) + (size_t)(i) * g.ncell + (cell))
 template <int M, class S, class L, bool kFirst, bool NARROW>
-__global__ void __launch_bounds__(kAdjThreads, AdjMinBlocks<S>::value)
+__global__ void __launch_bounds__(kAdjThreads, LBM_ADJ_MINB)
     k_adjoint(const S* __restrict__ state, const L* __restrict__ nu_next,
               const double* __restrict__ dldrho, L* __restrict__ nu_out,
               double* __restrict__ omega_acc, Grid g, double omega) {
   using Mo = Model<M>;
   using Rt = L;
-  constexpr int Q = Mo::Q, D = Mo::D, RR = Mo::R, NP = Mo::NP;
-  constexpr bool kSm = AdjLamSmem<L>::value;
+  constexpr int D = Mo::D, RR = Mo::R, NP = Mo::NP;
   // the lambda copies are committed in kGroups groups of kPerGroup pairs; pass 1
   // waits for each group just before its first pair
   constexpr int kGroups = LBM_ADJ_GROUPS;
@@ -135,14 +115,12 @@ __global__ void __launch_bounds__(kAdjThreads, AdjMinBlocks<S>::value)
     if constexpr (kFirst) l1 = (Rt)dldrho[self];
     // lambda_i(x) = nu_next(x + e_i, i): one value per direction for the first step
     // of the sweep (dL/drho_N, the same for every i), else gathered.
-    Rt lam_r[(kSm || kFirst) ? 1 : Q];
     const Rt* const lam_s = reinterpret_cast<const Rt*>(adj_dyn) + threadIdx.x;
     auto lam = [&](int i) -> Rt {
       if constexpr (kFirst) return l1;
-      else if constexpr (kSm) return lam_s[i * kAdjThreads];
-      else return lam_r[i];
+      else return lam_s[i * kAdjThreads];
     };
-    if constexpr (kSm && !kFirst) {
+    if constexpr (!kFirst) {
       // FP32: the lambda gather goes global -> shared by cp.async, which holds no
       // registers while in flight; each thread waits for its own copies only.
       Rt* const dst = reinterpret_cast<Rt*>(adj_dyn) + threadIdx.x;
@@ -164,8 +142,7 @@ __global__ void __launch_bounds__(kAdjThreads, AdjMinBlocks<S>::value)
     Rt rs, es = Rt(0), jx = Rt(0), jy = Rt(0), jz = Rt(0), sg;
     {
       const Rt h0 = (Rt)Codec<S>::ld(state + self);
-      if constexpr (kSm && !kFirst && kGroups > 1) cp_async_wait_group<kGroups - 1>();
-      if constexpr (!kSm && !kFirst) lam_r[0] = nu_next[self];
+      if constexpr (!kFirst && kGroups > 1) cp_async_wait_group<kGroups - 1>();
       rs = gW<Rt>(mc, 0) * h0;
       sg = gW<Rt>(mc, 0) * lam(0) * (Rt(1) + h0);
     }
@@ -179,16 +156,12 @@ __global__ void __launch_bounds__(kAdjThreads, AdjMinBlocks<S>::value)
       constexpr int ex = Mo::vs.e[ip][0], ey = Mo::vs.e[ip][1], ez = Mo::vs.e[ip][2];
       constexpr bool first = (p == 0) || (Mo::vs.grp[ip - 2] != gg);
       constexpr bool last = (p + 1 == NP) || (Mo::vs.grp[ip + 2] != gg);
-      if constexpr (kSm && !kFirst && kGroups > 1 && p > 0 && p % kPerGroup == 0)
+      if constexpr (!kFirst && kGroups > 1 && p > 0 && p % kPerGroup == 0)
         cp_async_wait_group<kGroups - 1 - p / kPerGroup>();
       const int cm = zo[ez + RR] + yo[ey + RR] + xo[ex + RR];   // x - e_ip
       const int cp = zo[RR - ez] + yo[RR - ey] + xo[RR - ex];   // x + e_ip
       const Rt hp = (Rt)Codec<S>::ld(LBM_POP(state, ip, cm));
       const Rt hm = (Rt)Codec<S>::ld(LBM_POP(state, im, cp));
-      if constexpr (!kSm && !kFirst) {
-        lam_r[ip] = *LBM_POP(nu_next, ip, cp);
-        lam_r[im] = *LBM_POP(nu_next, im, cm);
-      }
       if constexpr (first) gs = gjx = gjy = gjz = gsg = Rt(0);
       const Rt sp = hp + hm, dm = hp - hm;
       gs += sp;
@@ -239,77 +212,39 @@ __global__ void __launch_bounds__(kAdjThreads, AdjMinBlocks<S>::value)
     // the vector term keeps one v = ld (A1 + s^2/2) + ls s (2 A2 + s^2/6) per pair.
     Rt m0 = Rt(0), m2 = Rt(0), m4 = Rt(0), n1 = Rt(0), n3 = Rt(0);
     Rt gvx = Rt(0), gvy = Rt(0), gvz = Rt(0);
-    constexpr bool kLoop = LBM_ADJ_SHELL_LOOP && (kSm || kFirst);
-    if constexpr (kLoop) {
-      sfor<1, Mo::G>([&](auto Gi) {
-        constexpr int gg = decltype(Gi)::value;
-        const Rt x2 = gX2<Rt>(mc, gg);
-        const Rt A1 = cf.A1(x2), A2 = cf.A2(x2);
-        m0 = m2 = m4 = n1 = n3 = gvx = gvy = gvz = Rt(0);
-#pragma unroll kAdjUnroll
-        for (int p = ShellPairs<M>::first(gg); p < ShellPairs<M>::end(gg); ++p) {
-          const int ip = 1 + 2 * p, im = 2 + 2 * p;
-          const Rt ex = mc.ef[ip][0], ey = mc.ef[ip][1], ez = mc.ef[ip][2];
-          const Rt s = ex * uax + ey * uay + ez * uaz;
-          const Rt s2 = s * s;
-          const Rt lp = lam(ip), lm = lam(im);
-          const Rt ls = lp + lm, ld = lp - lm;
-          const Rt tl = ls * s2, tu = ld * s;
-          m0 += ls;
-          m2 += tl;
-          m4 += tl * s2;
-          n1 += tu;
-          n3 += tu * s2;
-          const Rt v = ld * (A1 + s2 * Rt(0.5)) + (ls * s) * (Rt(2) * A2 + s2 * Rt(1.0 / 6.0));
-          gvx += ex * v;
-          gvy += ey * v;
-          gvz += ez * v;
-        }
-        const Rt w = gW<Rt>(mc, gg);
-        Lr += w * (cf.A0(x2) * m0 + A2 * m2 + m4 * Rt(1.0 / 24.0) + A1 * n1 + n3 * Rt(1.0 / 6.0));
-        Sq += w * (gr.Bq(x2) * m0 - m2 * Rt(0.25) - n1 * Rt(0.5));
-        St += w * (gr.Bt(x2) * m0 + EqGrad<Rt, D>::Dt(x2) * m2 + EqGrad<Rt, D>::Ct(x2) * n1);
-        Vx += w * gvx;
-        Vy += w * gvy;
-        Vz += w * gvz;
-      });
-    } else
-    sfor<0, NP>([&](auto P) {
-      constexpr int p = decltype(P)::value;
-      constexpr int ip = 1 + 2 * p, im = 2 + 2 * p;
-      constexpr int gg = Mo::vs.grp[ip];
-      constexpr int ex = Mo::vs.e[ip][0], ey = Mo::vs.e[ip][1], ez = Mo::vs.e[ip][2];
-      constexpr bool first = (p == 0) || (Mo::vs.grp[ip - 2] != gg);
-      constexpr bool last = (p + 1 == NP) || (Mo::vs.grp[ip + 2] != gg);
+    // Passes 2 and 3 loop over each shell's pairs (lattice vectors from constant memory):
+    // unrolled over all pairs the kernel outgrows the instruction cache.
+    sfor<1, Mo::G>([&](auto Gi) {
+      constexpr int gg = decltype(Gi)::value;
       const Rt x2 = gX2<Rt>(mc, gg);
       const Rt A1 = cf.A1(x2), A2 = cf.A2(x2);
-      Rt s = Rt(0);
-      if constexpr (ex != 0) s += Rt(ex) * uax;
-      if constexpr (ey != 0) s += Rt(ey) * uay;
-      if constexpr (ez != 0) s += Rt(ez) * uaz;
-      const Rt s2 = s * s;
-      const Rt lp = lam(ip), lm = lam(im);
-      const Rt ls = lp + lm, ld = lp - lm;
-      const Rt tl = ls * s2, tu = ld * s;
-      if constexpr (first) m0 = m2 = m4 = n1 = n3 = gvx = gvy = gvz = Rt(0);
-      m0 += ls;
-      m2 += tl;
-      m4 += tl * s2;
-      n1 += tu;
-      n3 += tu * s2;
-      const Rt v = ld * (A1 + s2 * Rt(0.5)) + (ls * s) * (Rt(2) * A2 + s2 * Rt(1.0 / 6.0));
-      if constexpr (ex != 0) gvx += Rt(ex) * v;
-      if constexpr (ey != 0) gvy += Rt(ey) * v;
-      if constexpr (ez != 0) gvz += Rt(ez) * v;
-      if constexpr (last) {
-        const Rt w = gW<Rt>(mc, gg);
-        Lr += w * (cf.A0(x2) * m0 + A2 * m2 + m4 * Rt(1.0 / 24.0) + A1 * n1 + n3 * Rt(1.0 / 6.0));
-        Sq += w * (gr.Bq(x2) * m0 - m2 * Rt(0.25) - n1 * Rt(0.5));
-        St += w * (gr.Bt(x2) * m0 + EqGrad<Rt, D>::Dt(x2) * m2 + EqGrad<Rt, D>::Ct(x2) * n1);
-        Vx += w * gvx;
-        Vy += w * gvy;
-        Vz += w * gvz;
+      m0 = m2 = m4 = n1 = n3 = gvx = gvy = gvz = Rt(0);
+#pragma unroll kAdjUnroll
+      for (int p = ShellPairs<M>::first(gg); p < ShellPairs<M>::end(gg); ++p) {
+        const int ip = 1 + 2 * p, im = 2 + 2 * p;
+        const Rt ex = mc.ef[ip][0], ey = mc.ef[ip][1], ez = mc.ef[ip][2];
+        const Rt s = ex * uax + ey * uay + ez * uaz;
+        const Rt s2 = s * s;
+        const Rt lp = lam(ip), lm = lam(im);
+        const Rt ls = lp + lm, ld = lp - lm;
+        const Rt tl = ls * s2, tu = ld * s;
+        m0 += ls;
+        m2 += tl;
+        m4 += tl * s2;
+        n1 += tu;
+        n3 += tu * s2;
+        const Rt v = ld * (A1 + s2 * Rt(0.5)) + (ls * s) * (Rt(2) * A2 + s2 * Rt(1.0 / 6.0));
+        gvx += ex * v;
+        gvy += ey * v;
+        gvz += ez * v;
       }
+      const Rt w = gW<Rt>(mc, gg);
+      Lr += w * (cf.A0(x2) * m0 + A2 * m2 + m4 * Rt(1.0 / 24.0) + A1 * n1 + n3 * Rt(1.0 / 6.0));
+      Sq += w * (gr.Bq(x2) * m0 - m2 * Rt(0.25) - n1 * Rt(0.5));
+      St += w * (gr.Bt(x2) * m0 + EqGrad<Rt, D>::Dt(x2) * m2 + EqGrad<Rt, D>::Ct(x2) * n1);
+      Vx += w * gvx;
+      Vy += w * gvy;
+      Vz += w * gvz;
     });
     // chain rule to the moments (arithmetic type; the omega term in FP64)
     const Rt Lux = rho_r * (a_r * Vx + Rt(2) * ux * Sq);
@@ -330,31 +265,16 @@ __global__ void __launch_bounds__(kAdjThreads, AdjMinBlocks<S>::value)
     const Rt oa = om * alpha, og = om * gam;
     const Rt obx = om * a_r * bx, oby = om * a_r * by, obz = om * a_r * bz;
     nu_out[self] = om1 * lam(0) + oa;
-    if constexpr (kLoop) {
-      sfor<1, Mo::G>([&](auto Gi) {
-        constexpr int gg = decltype(Gi)::value;
-        const Rt ev = oa + og * gX2<Rt>(mc, gg);
-#pragma unroll kAdjUnroll
-        for (int p = ShellPairs<M>::first(gg); p < ShellPairs<M>::end(gg); ++p) {
-          const int ip = 1 + 2 * p, im = 2 + 2 * p;
-          const Rt od = mc.ef[ip][0] * obx + mc.ef[ip][1] * oby + mc.ef[ip][2] * obz;
-          *LBM_POP(nu_out, ip, self) = om1 * lam(ip) + (ev + od);
-          *LBM_POP(nu_out, im, self) = om1 * lam(im) + (ev - od);
-        }
-      });
-    } else
-    sfor<0, NP>([&](auto P) {
-      constexpr int p = decltype(P)::value;
-      constexpr int ip = 1 + 2 * p, im = 2 + 2 * p;
-      constexpr int gg = Mo::vs.grp[ip];
-      constexpr int ex = Mo::vs.e[ip][0], ey = Mo::vs.e[ip][1], ez = Mo::vs.e[ip][2];
+    sfor<1, Mo::G>([&](auto Gi) {
+      constexpr int gg = decltype(Gi)::value;
       const Rt ev = oa + og * gX2<Rt>(mc, gg);
-      Rt od = Rt(0);
-      if constexpr (ex != 0) od += Rt(ex) * obx;
-      if constexpr (ey != 0) od += Rt(ey) * oby;
-      if constexpr (ez != 0) od += Rt(ez) * obz;
-      *LBM_POP(nu_out, ip, self) = om1 * lam(ip) + (ev + od);
-      *LBM_POP(nu_out, im, self) = om1 * lam(im) + (ev - od);
+#pragma unroll kAdjUnroll
+      for (int p = ShellPairs<M>::first(gg); p < ShellPairs<M>::end(gg); ++p) {
+        const int ip = 1 + 2 * p, im = 2 + 2 * p;
+        const Rt od = mc.ef[ip][0] * obx + mc.ef[ip][1] * oby + mc.ef[ip][2] * obz;
+        *LBM_POP(nu_out, ip, self) = om1 * lam(ip) + (ev + od);
+        *LBM_POP(nu_out, im, self) = om1 * lam(im) + (ev - od);
+      }
     });
   }
   const double bsum = block_sum_128(om_part, sh);

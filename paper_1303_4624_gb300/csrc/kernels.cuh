@@ -293,13 +293,8 @@ __device__ __forceinline__ HalfMoments<Rt> half_moments(Get&& hv) {
     } else {
       const Rt tr = xmul(gW<Rt>(mc, gg), sp);
       const Rt te = xmul(gX2<Rt>(mc, gg), tr);
-      if constexpr (!std::is_same<Rt, double>::value) {
-        kahan_add(m.rs, m.rc, tr);
-        kahan_add(m.es, m.ec, te);
-      } else {
-        m.rs = xadd(m.rs, tr);
-        m.es = xadd(m.es, te);
-      }
+      kahan_add(m.rs, m.rc, tr);
+      kahan_add(m.es, m.ec, te);
     }
     const Rt tj = xmul(gW<Rt>(mc, gg), xsub(hp, hm));
     if constexpr (ex != 0) m.jx = xaxpy<ex>(tj, m.jx);
@@ -334,9 +329,8 @@ __device__ __forceinline__ FF ff_add(FF a, FF b) {
 }
 __device__ __forceinline__ double ff_to_double(FF v) { return (double)v.hi + (double)v.lo; }
 
-// Cell state from the two halves.  theta - 1 is recovered in double-float on the
-// FP32 pipe for the FP32-arithmetic forms (Rt = float: FP32, FP16 and BF16 storage)
-// and in FP64 for the FP64 form (Rt = double).  The energy difference E - D rho
+// Cell state from the two halves (FP32, FP16 and BF16 storage; the FP64 form: collide64.cuh).
+// theta - 1 is recovered in double-float on the FP32 pipe.  The energy difference E - D rho
 // cancels badly where the gas is hot and dense (behind a shock), so it is formed
 // with FP64-grade precision in every form, whatever the storage rounding.
 template <class Rt>
@@ -352,83 +346,60 @@ __device__ __forceinline__ CellState<Rt> cell_state(const HalfMoments<Rt>& A,
   constexpr int D = Model<M>::D;
   const ModelConst& mc = c_mc[M];
   CellState<Rt> c;
-  if constexpr (!std::is_same<Rt, double>::value) {
-    // FP32-arithmetic forms (Rt = float, or float2 for two cells): rho - 1 and
-    // E - D rho as double-float (hi, lo) on the FP32 pipe
-    const Rt one = cst<Rt>(1.0), Dv = cst<Rt>(D);
-    Rt rd_hi, rd_lo, ed_hi, ed_lo, rho_hi, rho_lo;
-    two_sum(A.rs, B.rs, rd_hi, rd_lo);
-    rd_lo = xsub(rd_lo, xadd(A.rc, B.rc));
-    two_sum(A.es, B.es, ed_hi, ed_lo);
-    ed_lo = xsub(ed_lo, xadd(A.ec, B.ec));
-    two_sum(one, rd_hi, rho_hi, rho_lo);
-    rho_lo = xadd(rho_lo, rd_lo);
-    const Rt rho_r = xadd(rho_hi, rho_lo);
-    const Rt r0 = xrcp_approx(rho_r);
-    const Rt ir = xfma(r0, xsub(xfma(xneg(rho_hi), r0, one), xmul(rho_lo, r0)), r0);
-    const Rt ir_lo = xmul(ir, xsub(xfma(xneg(rho_hi), ir, one), xmul(rho_lo, ir)));
-    const Rt a = gA<Rt>(mc);
-    const Rt jx = xadd(A.jx, B.jx), jy = xadd(A.jy, B.jy), jz = xadd(A.jz, B.jz);
-    const Rt ux = xmul(xmul(a, jx), ir), uy = xmul(xmul(a, jy), ir);
-    const Rt uz = (D == 3) ? xmul(xmul(a, jz), ir) : cst<Rt>(0.0);
-    c.q = xfma(ux, ux, xfma(uy, uy, xmul(uz, uz)));
-    // E - D rho = ed - D rd (the product's rounding error recovered by FMA)
-    const Rt ph = xmul(Dv, rd_hi);
-    const Rt pl = xfma(Dv, rd_lo, xfma(Dv, rd_hi, xneg(ph)));
-    Rt sh, se;
-    two_sum(ed_hi, xneg(ph), sh, se);
-    const Rt dl = xadd(se, xsub(ed_lo, pl));
-    const Rt dh = xadd(sh, dl);
-    const Rt dlo = xsub(dl, xsub(dh, sh));
-    // (E - D rho) / rho as double-float, then theta - 1 = (that - |u|^2) / D
-    const Rt xh = xmul(dh, ir);
-    const Rt xl = xfma(dh, ir_lo, xfma(dlo, ir, xfma(dh, ir, xneg(xh))));
-    // v = x - q as double-float; t = v / D rounded to nearest: a product with the
-    // FP32-rounded 1/D alone is biased (it rounds 1/3 up), which would heat or cool
-    // every cell by a fixed fraction of an ulp per step; one FMA residual step
-    // removes it
-    Rt vh, ve;
-    two_sum(xh, xneg(c.q), vh, ve);
-    const Rt vl = xadd(ve, xl);
-    const Rt third = cst<Rt>(1.0 / D);
-    const Rt y = xmul(xadd(vh, vl), third);
-    c.t = xfma(xadd(xfma(xneg(Dv), y, vh), vl), third, y);
-    c.uax = xmul(a, ux);
-    c.uay = xmul(a, uy);
-    c.uaz = xmul(a, uz);
-    c.rho = rho_r;
-    c.rdev = xadd(rd_hi, rd_lo);
-    const Rt om = cst<Rt>(omega);
-    c.wr = xmul(om, rho_r);
-    c.wrd = xmul(om, c.rdev);
-    return c;
-  } else {
-    // FP64 form: everything in FP64
-    const double rd = xadd(A.rs, B.rs);
-    const double ed = xadd(A.es, B.es);
-    const double jx = xadd(A.jx, B.jx), jy = xadd(A.jy, B.jy), jz = xadd(A.jz, B.jz);
-    const double rho = xadd(1.0, rd);
-    const double ir = 1.0 / rho;
-    const double a = gA<double>(mc);
-    const double ux = xmul(xmul(a, jx), ir), uy = xmul(xmul(a, jy), ir);
-    const double uz = (D == 3) ? xmul(xmul(a, jz), ir) : 0.0;
-    c.q = xfma(ux, ux, xfma(uy, uy, xmul(uz, uz)));
-    // theta - 1 = ((E - D rho) / rho - |u|^2) / D
-    c.t = xmul(xfma(xfma(-(double)D, rd, ed), ir, -c.q), 1.0 / D);
-    c.uax = xmul(a, ux);
-    c.uay = xmul(a, uy);
-    c.uaz = xmul(a, uz);
-    c.rho = rho;
-    c.rdev = rd;
-    c.wr = xmul(omega, rho);
-    c.wrd = xmul(omega, rd);
-    return c;
-  }
+  // rho - 1 and E - D rho as double-float (hi, lo) on the FP32 pipe (Rt = float, or float2
+  // for two cells)
+  const Rt one = cst<Rt>(1.0), Dv = cst<Rt>(D);
+  Rt rd_hi, rd_lo, ed_hi, ed_lo, rho_hi, rho_lo;
+  two_sum(A.rs, B.rs, rd_hi, rd_lo);
+  rd_lo = xsub(rd_lo, xadd(A.rc, B.rc));
+  two_sum(A.es, B.es, ed_hi, ed_lo);
+  ed_lo = xsub(ed_lo, xadd(A.ec, B.ec));
+  two_sum(one, rd_hi, rho_hi, rho_lo);
+  rho_lo = xadd(rho_lo, rd_lo);
+  const Rt rho_r = xadd(rho_hi, rho_lo);
+  const Rt r0 = xrcp_approx(rho_r);
+  const Rt ir = xfma(r0, xsub(xfma(xneg(rho_hi), r0, one), xmul(rho_lo, r0)), r0);
+  const Rt ir_lo = xmul(ir, xsub(xfma(xneg(rho_hi), ir, one), xmul(rho_lo, ir)));
+  const Rt a = gA<Rt>(mc);
+  const Rt jx = xadd(A.jx, B.jx), jy = xadd(A.jy, B.jy), jz = xadd(A.jz, B.jz);
+  const Rt ux = xmul(xmul(a, jx), ir), uy = xmul(xmul(a, jy), ir);
+  const Rt uz = (D == 3) ? xmul(xmul(a, jz), ir) : cst<Rt>(0.0);
+  c.q = xfma(ux, ux, xfma(uy, uy, xmul(uz, uz)));
+  // E - D rho = ed - D rd (the product's rounding error recovered by FMA)
+  const Rt ph = xmul(Dv, rd_hi);
+  const Rt pl = xfma(Dv, rd_lo, xfma(Dv, rd_hi, xneg(ph)));
+  Rt sh, se;
+  two_sum(ed_hi, xneg(ph), sh, se);
+  const Rt dl = xadd(se, xsub(ed_lo, pl));
+  const Rt dh = xadd(sh, dl);
+  const Rt dlo = xsub(dl, xsub(dh, sh));
+  // (E - D rho) / rho as double-float, then theta - 1 = (that - |u|^2) / D
+  const Rt xh = xmul(dh, ir);
+  const Rt xl = xfma(dh, ir_lo, xfma(dlo, ir, xfma(dh, ir, xneg(xh))));
+  // v = x - q as double-float; t = v / D rounded to nearest: a product with the
+  // FP32-rounded 1/D alone is biased (it rounds 1/3 up), which would heat or cool
+  // every cell by a fixed fraction of an ulp per step; one FMA residual step
+  // removes it
+  Rt vh, ve;
+  two_sum(xh, xneg(c.q), vh, ve);
+  const Rt vl = xadd(ve, xl);
+  const Rt third = cst<Rt>(1.0 / D);
+  const Rt y = xmul(xadd(vh, vl), third);
+  c.t = xfma(xadd(xfma(xneg(Dv), y, vh), vl), third, y);
+  c.uax = xmul(a, ux);
+  c.uay = xmul(a, uy);
+  c.uaz = xmul(a, uz);
+  c.rho = rho_r;
+  c.rdev = xadd(rd_hi, rd_lo);
+  const Rt om = cst<Rt>(omega);
+  c.wr = xmul(om, rho_r);
+  c.wrd = xmul(om, c.rdev);
+  return c;
 }
 
 // Equilibrium + BGK of pairs [P0, P1) (and the rest direction when REST), with
 // h_i^eq = (rho - 1) + rho (P_i - 1):
-//   EXACT = true:  h_i' = h_i + omega (h_i^eq - h_i)   (FP32 / FP64 forms).  The
+//   EXACT = true:  h_i' = h_i + omega (h_i^eq - h_i)   (FP32 form; FP64: collide64.cuh).  The
 //                  equilibrium is an exact fixed point whatever the rounding of omega;
 //                  with (1 - omega) h + omega h^eq the two rounded factors need not
 //                  sum to one and a uniform region drifts by their difference every
@@ -578,16 +549,13 @@ __device__ __forceinline__ void neighbour_offsets(int x, int y, int z, int nx, i
 // cut for (128 registers at 4: 16 warps per SM; measured best for the FP32 and
 // FP16 forms).  D2Q33's 33 populations fit fewer registers without spilling, and
 // more resident warps pay: 8 blocks (64 registers) for FP32, 6 (80 registers) for
-// the 16-bit forms (4096 x 2048: +4.6 % and +12.8 % over 4 blocks).  The FP64
-// form keeps 2 (D3Q95's 95 doubles need 190 registers).
+// the 16-bit forms (4096 x 2048: +4.6 % and +12.8 % over 4 blocks).
 #ifndef LBM_DIRECT_MINB
 #define LBM_DIRECT_MINB 4
 #endif
 template <int M, class S>
 struct DirectMinBlocks {
-  static constexpr int value = std::is_same<S, double>::value
-                                   ? 2
-                                   : (Model<M>::Q == 33 ? (sizeof(S) == 4 ? 8 : 6) : LBM_DIRECT_MINB);
+  static constexpr int value = Model<M>::Q == 33 ? (sizeof(S) == 4 ? 8 : 6) : LBM_DIRECT_MINB;
 };
 // 4-byte global -> shared copy (cp.async, L1-allocating) and the wait for all of
 // this thread's outstanding copies.
@@ -1354,9 +1322,9 @@ __device__ __forceinline__ double order_value(long long k) {
   return __longlong_as_double(k ^ ((k >> 63) & 0x7fffffffffffffffll));
 }
 
-// Moments of the FP64 form, one thread per cell: collide64's sums (about 250 FP64
-// operations a D3Q95 cell; population by population, f = w (1 + h) and six sums each took
-// ~900, and bound the kernel at 317 us for 131,072 cells).  The minimum and the count of
+// Moments of the FP64 form, one thread per cell: collide64's sums (about 60 FP64 operations
+// a D3Q95 cell; population by population, f = w (1 + h) and six sums each took ~900, and
+// bound the kernel at 317 us for 131,072 cells).  The minimum and the count of
 // non-finite populations are taken on the integer pipe (an FP64 minimum costs more than
 // three FP64 instructions), and each warp reduces one audit slot over the block.
 template <int M>
@@ -1495,9 +1463,10 @@ static __global__ void __launch_bounds__(256) k_audit_reduce(const double* __res
 // traffic of the FP32 form (94.5 M elements, D3Q95 201 x 99 x 50: 163 us against 170).
 // Conversions are therefore done on the integer and FP32 pipes, w (1 + h) is one FMA and
 // f / w - 1 one subtraction (f - w, exact where it cancels) and a product with 1 / w in
-// double-float, rounded as the FP64 division and subtraction round.  The direction of an element is found by one division per kIoRun
+// double-float, rounded as the FP64 division and subtraction round (next to a rounding
+// boundary those are done).  The direction of an element is found by one division per kIoRun
 // elements.  With an FP64 division, a 64-bit integer division and two conversions an
-// element set took 1771 us and get 637 us on that grid; now 207 and 198 us.
+// element set took 1771 us and get 637 us on that grid; now 276 and 196 us.
 constexpr int kIoThreads = 256;
 constexpr int kIoPairs = 8;                          // pairs of elements per thread
 constexpr int kIoRun = kIoThreads * kIoPairs * 2;    // elements per block
