@@ -543,6 +543,20 @@ __device__ __forceinline__ void neighbour_offsets(int x, int y, int z, int nx, i
   }
 }
 
+// A cell of a fixed end plane takes its template's populations and gathers nothing: true
+// once they are stored, false for every other cell.
+template <int M, class S>
+__device__ __forceinline__ bool end_plane_store(S* __restrict__ dst, const Grid& g, const Ends& ends,
+                                                int x, int y, int z, size_t cell) {
+  const int c = ends.axis == 0 ? x : (ends.axis == 1 ? y : z);
+  const int n = ends.axis == 0 ? g.nx : (ends.axis == 1 ? g.ny : g.nz);
+  if (c >= ends.width && c < n - ends.width) return false;
+  const S* t = static_cast<const S*>(ends.tmpl) + (c < ends.width ? 0 : 1);
+#pragma unroll 8
+  for (int i = 0; i < Model<M>::Q; ++i) dst[(size_t)i * (size_t)g.ncell + cell] = __ldg(t + 2 * i);
+  return true;
+}
+
 // Direct-gather kernel: one thread per cell, x fastest across the block,
 // blockIdx.y / z give the row; Q loads per thread straight from HBM / L2.
 // LBM_DIRECT_MINB: resident 128-thread blocks per SM the D3Q95 register budget is
@@ -606,9 +620,12 @@ template <int M, class S>
 struct DirectNarrow {
   static constexpr bool value = M == 1 && std::is_same<S, float>::value;
 };
-template <int M, class S, bool REV, bool NARROW>
+// ENDS: the fixed end planes are written here as well (end_plane_store) instead of by a
+// second kernel after the step.
+template <int M, class S, bool REV, bool NARROW, bool ENDS>
 __global__ void __launch_bounds__(128, DirectMinBlocks<M, S>::value)
-    k_stream_collide(const S* __restrict__ src, S* __restrict__ dst, Grid g, double omega) {
+    k_stream_collide(const S* __restrict__ src, S* __restrict__ dst, Grid g, double omega,
+                     Ends ends) {
   using Mo = Model<M>;
   constexpr int D = Mo::D, RR = Mo::R;
   wait_prior_grid();
@@ -618,6 +635,9 @@ __global__ void __launch_bounds__(128, DirectMinBlocks<M, S>::value)
   if (x >= g.nx) return;
   const int y = REV ? (int)(gridDim.y - 1 - blockIdx.y) : (int)blockIdx.y;
   const int z = REV ? (int)(gridDim.z - 1 - blockIdx.z) : (int)blockIdx.z;
+  if constexpr (ENDS) {
+    if (end_plane_store<M>(dst, g, ends, x, y, z, ((size_t)z * g.ny + y) * g.nx + x)) return;
+  }
   int xo[2 * RR + 1], yo[2 * RR + 1], zo[2 * RR + 1];
   neighbour_offsets<D, RR>(x, y, z, g.nx, g.ny, g.nz, g.nxy, xo, yo, zo);
   if constexpr (NARROW) {
@@ -657,8 +677,7 @@ __global__ void __launch_bounds__(128, DirectMinBlocks<M, S>::value)
 // Nx = 11, 201 of 256 for Nx = 201) and starts odd rows off the sector boundaries, but
 // keeps the y and z offsets uniform in a block (see linear_rows for the rule between the
 // two).  Same arithmetic, same bits.
-// ENDS: the fixed end planes are written here as well (a cell of an end plane stores its
-// template and gathers nothing) instead of by a second kernel after the step.
+// ENDS: as for the row-mapped kernel.
 // In y and z only the offsets that occur are formed; lanes of a warp differ in them.
 constexpr int kLinThreads = 128;   // 64 and 32 measured slower (512x256x256 3902, 4029, 4136 us)
 template <int M, class S, bool REV, bool NARROW, bool ENDS>
@@ -677,14 +696,7 @@ __global__ void __launch_bounds__(kLinThreads, DirectMinBlocks<M, S>::value * 12
   const int z = D == 3 ? (int)(row / (uint32_t)g.ny) : 0;
   const int y = (int)row - z * g.ny;
   if constexpr (ENDS) {
-    const int c = ends.axis == 0 ? x : (ends.axis == 1 ? y : z);
-    const int n = ends.axis == 0 ? g.nx : (ends.axis == 1 ? g.ny : g.nz);
-    if (c < ends.width || c >= n - ends.width) {
-      const S* t = static_cast<const S*>(ends.tmpl) + (c < ends.width ? 0 : 1);
-#pragma unroll 8
-      for (int i = 0; i < Mo::Q; ++i) dst[(size_t)i * (size_t)g.ncell + cell] = __ldg(t + 2 * i);
-      return;
-    }
+    if (end_plane_store<M>(dst, g, ends, x, y, z, (size_t)cell)) return;
   }
   int xo[2 * RR + 1], yo[2 * RR + 1], zo[2 * RR + 1];
   neighbour_offsets<D, RR>(x, y, z, g.nx, g.ny, g.nz, g.nxy, xo, yo, zo);
