@@ -231,10 +231,12 @@ __device__ __forceinline__ Cell64 cell64(const Mom64& m) {
 }
 
 // h + omega (h^eq - h) of a pair's two members, h^eq = ev +- od: in fixed point at the
-// scale of the largest of the four terms (140 integer instructions for six at the FP64
-// rate); om is omega in units of 2^-62.  The error is a few units of 2^-60 of that term,
-// against omega 2^-53 of it in FP64; a smaller omega than 2^-6 (0 must return h as it is)
-// keeps the FP64 operations.
+// scale of the largest of the four terms (about 160 integer instructions for six at the FP64
+// rate); om is omega in units of 2^-62.  The error is at most nine units of 2^-60 of that
+// term's power of two (five from the terms' truncation, four from the product), without a
+// preferred sign, against omega 2^-53 of it in FP64; a smaller omega than 2^-6 (0 must
+// return h as it is) keeps the FP64 operations (tested on om: an FP64 comparison would cost
+// as much as an addition).
 struct Two64 {
   double p, m;
 };
@@ -246,12 +248,12 @@ static __device__ __noinline__ Two64 relax_pair_any(double ev, double od, double
 static __device__ __noinline__ Two64 relax_pair64(double ev, double od, double hp, double hm,
                                               double omega, long long om) {
   const int top = max(max(fx_top(ev), fx_top(od)), max(fx_top(hp), fx_top(hm)));
-  if (!fx_regular(top) || omega < 0x1p-6) return relax_pair_any(ev, od, hp, hm, omega);
+  if (!fx_regular(top) || om < (1ll << 56)) return relax_pair_any(ev, od, hp, hm, omega);
   const int e = fx_exponent(top);
   const long long v = fx_from<60>(ev, e), o = fx_from<60>(od, e);
   const long long p = fx_from<60>(hp, e), m = fx_from<60>(hm, e);
   // |v + o - p| < 3 2^60; times omega < 2: below 6 2^60
-  return {fx_to<60>(p + 4 * fx_mulhi(v + o - p, om), e), fx_to<60>(m + 4 * fx_mulhi(v - o - m, om), e)};
+  return {fx_to<60>(p + fx_mul(v + o - p, om), e), fx_to<60>(m + fx_mul(v - o - m, om), e)};
 }
 
 // The relaxation h' = h + omega (h^eq - h) of one part's pairs.

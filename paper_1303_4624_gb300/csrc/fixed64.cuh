@@ -10,14 +10,14 @@
 // top: the largest (high word & 0x7fffffff) of the group; its exponent field e bounds
 // |v| < 2^(e - 1022).  A value v is held as trunc(v 2^(B - (e - 1022))) with B bits.
 // Groups with an exponent field of 2000 or more (|v| >= 2^977, Inf, NaN) are the caller's
-// (fx_regular); fields below 128 count as 128 (|v| < 2^-894 is held as 0).
+// (fx_regular); fields below 64 count as 64 (|v| < 2^-1014 is held as 0).
 #pragma once
 
 namespace lbm {
 
 __device__ __forceinline__ int fx_top(double v) { return __double2hiint(v) & 0x7fffffff; }
 __device__ __forceinline__ bool fx_regular(int top) { return top < (2000 << 20); }
-__device__ __forceinline__ int fx_exponent(int top) { return max(top >> 20, 128); }
+__device__ __forceinline__ int fx_exponent(int top) { return max(top >> 20, 64); }
 
 // v with B bits below 2^(e - 1022): 63 - B + e(v)'s distance is the right shift.
 template <int B>
@@ -29,25 +29,35 @@ __device__ __forceinline__ long long fx_from(double v, int e) {
   const long long s = (long long)((int)h >> 31);
   return ((long long)(m >> r) ^ s) - s;
 }
-// The double nearest to i (B bits below 2^(e - 1022)).
+// The double nearest to i (B bits below 2^(e - 1022)), of two equally near ones the even: a
+// sum of doubles of one exponent has a few bits more than 53 and often ends in a tie, which
+// must not always go the same way (away from zero, it cost a relaxing flow 4e-18 of its mass
+// a step).
 template <int B>
 __device__ __forceinline__ double fx_to(long long i, int e) {
   const long long s = i >> 63;
   const unsigned long long u = (unsigned long long)((i ^ s) - s);
   const int lz = __clzll((long long)u);
   const unsigned long long m = u << (lz & 63);
-  const unsigned long long f = (m >> 11) + ((m >> 10) & 1);   // 53 bits, rounded
+  const unsigned low = (unsigned)m;
+  const unsigned up = ((low & 0x7ffu) + 0x3ffu + ((low >> 11) & 1u)) >> 11;
+  const unsigned long long f = (m >> 11) + up;                // 53 bits, rounded
   const int exponent = e + (63 - B) + 1 - lz;                 // field of the leading bit
   unsigned long long bits = ((unsigned long long)(unsigned)(exponent - 1) << 52) + f;
   bits |= (unsigned long long)s & 0x8000000000000000ull;
   return __longlong_as_double(u == 0 ? 0ll : (long long)bits);
 }
-// a b / 2^64 to within three units, |a|, |b| < 2^63: three wide products.
-__device__ __forceinline__ long long fx_mulhi(long long a, long long b) {
-  const int ah = (int)(a >> 32), bh = (int)(b >> 32);
-  const int al = (int)((unsigned)a >> 1), bl = (int)((unsigned)b >> 1);
-  const long long t = (long long)ah * bl + (long long)al * bh;
-  return (long long)ah * bh + (t >> 31);
+// a f / 2^62 for |a| < 2^62 and an even factor f in [0, 2^63), |a f| < 2^125: three wide
+// products of the halves ah, al (a = 2^32 ah + 2 al + its lowest bit) and fh, fl.  Left out
+// are al fl, below four units, and the bits below a unit; `half` is their mean for this f
+// (al anywhere in its range) and ties go by al's last bit, so that the error, within four
+// units, has no preferred sign: a relaxation repeated at one omega would add it up.
+__device__ __forceinline__ long long fx_mul(long long a, long long f) {
+  const int fh = (int)(f >> 32), fl = (int)((unsigned)f >> 1);
+  const int ah = (int)(a >> 32), al = (int)((unsigned)a >> 1), a0 = (int)a & 1;
+  const int half = (1 << 28) + (fl >> 1) - (al & 1);
+  const long long t = (long long)ah * fl + ((long long)al * fh + ((long long)a0 * (fh >> 1) + half));
+  return (long long)ah * fh * 4 + (t >> 29);
 }
 
 }  // namespace lbm
