@@ -7,8 +7,7 @@
 // instruction count and not by memory: 1520 bytes a D3Q95 cell take 0.23 ns of HBM time,
 // the ~1290 FP64 operations of the pair-by-pair form 2.4 ns.  What brings D3Q95 to ~420:
 //   * moments shell by shell: the members of a shell share weight and |xi|^2, so their
-//     sums are formed unweighted (momentum in units of the primitive vector) and each
-//     shell is weighted once;
+//     sums are formed unweighted and each shell is weighted once;
 //   * those sums, and the relaxation's h + omega (h^eq - h), in 64-bit fixed point on the
 //     integer pipes (fixed64.cuh);
 //   * rho and rho - 1 folded into the shell's equilibrium coefficients, so a pair's
@@ -52,13 +51,6 @@ LBM_HD constexpr int shell_part64(int g) {
   return M == 0 ? d2[g] : d3[g];
 }
 
-template <int M>
-LBM_HD constexpr int shell_gcd(int g) {
-  for (int i = 1; i < Model<M>::Q; ++i)
-    if (Model<M>::vs.grp[i] == g)
-      return igcd(igcd(iabs(Model<M>::vs.e[i][0]), iabs(Model<M>::vs.e[i][1])), iabs(Model<M>::vs.e[i][2]));
-  return 0;
-}
 // Pairs [first, end) of symmetry group g (g >= 1) in storage order.
 template <int M>
 struct ShellPairs {
@@ -156,7 +148,6 @@ __device__ __forceinline__ Mom64 moments64(Get&& hv) {
     constexpr int g = decltype(Gi)::value;
     if constexpr (shell_part64<M>(g) == P) {
       constexpr int p0 = ShellPairs<M>::first(g), np = ShellPairs<M>::end(g) - p0;
-      constexpr int ge = shell_gcd<M>(g);
       double h[2 * np];
       int top = 0;
       sfor<0, 2 * np>([&](auto J) {
@@ -168,23 +159,24 @@ __device__ __forceinline__ Mom64 moments64(Get&& hv) {
       long long gs = 0, gx = 0, gy = 0, gz = 0;
       sfor<0, np>([&](auto J) {
         constexpr int j = decltype(J)::value, i = 1 + 2 * (p0 + j);
-        constexpr int bx = Mo::vs.e[i][0] / ge, by = Mo::vs.e[i][1] / ge, bz = Mo::vs.e[i][2] / ge;
+        constexpr int ex = Mo::vs.e[i][0], ey = Mo::vs.e[i][1], ez = Mo::vs.e[i][2];
         const SumDiff64 sd = sum_diff64(h[2 * j], h[2 * j + 1], e);
         const long long d = sd.d;
         gs += sd.s;
-        if constexpr (bx != 0) gx += bx * d;
-        if constexpr (by != 0) gy += by * d;
-        if constexpr (bz != 0) gz += bz * d;
+        if constexpr (ex != 0) gx += ex * d;
+        if constexpr (ey != 0) gy += ey * d;
+        if constexpr (ez != 0) gz += ez * d;
       });
       // sums: at most 72 2^56 < 2^63
       double S = fx_to<56>(gs, e), X = fx_to<56>(gx, e), Y = fx_to<56>(gy, e), Z = 0.0;
       if constexpr (Mo::D == 3) Z = fx_to<56>(gz, e);
       if (!fx_regular(top)) S = X = Y = Z = __longlong_as_double(0x7ff8000000000000ll);
-      m.r = none ? __dmul_rn(mc.W[g], S) : __fma_rn(mc.W[g], S, m.r);
-      m.e = none ? __dmul_rn(mc.WX2[g], S) : __fma_rn(mc.WX2[g], S, m.e);
-      m.x = none ? __dmul_rn(mc.Wk[g], X) : __fma_rn(mc.Wk[g], X, m.x);
-      m.y = none ? __dmul_rn(mc.Wk[g], Y) : __fma_rn(mc.Wk[g], Y, m.y);
-      if constexpr (Mo::D == 3) m.z = none ? __dmul_rn(mc.Wk[g], Z) : __fma_rn(mc.Wk[g], Z, m.z);
+      const double tr = __dmul_rn(mc.W[g], S);
+      m.r = none ? tr : __dadd_rn(m.r, tr);
+      m.e = none ? __dmul_rn(mc.X2[g], tr) : __fma_rn(mc.X2[g], tr, m.e);
+      m.x = none ? __dmul_rn(mc.W[g], X) : __fma_rn(mc.W[g], X, m.x);
+      m.y = none ? __dmul_rn(mc.W[g], Y) : __fma_rn(mc.W[g], Y, m.y);
+      if constexpr (Mo::D == 3) m.z = none ? __dmul_rn(mc.W[g], Z) : __fma_rn(mc.W[g], Z, m.z);
       none = false;
     }
   });
@@ -194,12 +186,17 @@ __device__ __forceinline__ Mom64 moments64(Get&& hv) {
 // What the relaxation needs of a cell: the velocity a u (s = e . v), and the equilibrium's
 // coefficients with rho folded in.  h^eq of a pair +- k b, with s = b . v, is
 //   c0 +- s c1 + s^2 c2 +- s^3 c3 + s^4 c4
-//   c0 = P0 + x2 K1 + (x2^2 / 8) tt,  c1 = k L0 + (k x2 / 2) rt,
-//   c2 = (k^2 / 2) d + (k^2 x2 / 4) rt,  c3 = (k^3 / 6) rho,  c4 = (k^4 / 24) rho
-// (EqCoef's polynomials times rho; rt = rho t, tt = rho t^2, d = L0 - rt).
+//   c0 = P0 + x2 (K1 + (x2 / 8) tt),  c1 = k (L0 + (x2 / 2) rt),
+//   c2 = k^2 (d2 + (x2 / 4) rt),  c3 = k^3 r6,  c4 = k^4 r24
+// (EqCoef's polynomials times rho; rt = rho t, tt = rho t^2, d2 = (L0 - rt) / 2, r6 = rho / 6,
+// r24 = rho / 24).  Of a shell only x2 (or an exact fraction of it), its weight and small
+// integers are multiplied in, as in the moments: a rounded product of them (W x2, k^3 / 6,
+// ...) is off by the same fraction of an ulp in every cell and step, and after 200 steps of
+// a 256 x 8 D2Q33 flow the populations' rms error was 4.8e-14 with such products, 1.6e-15
+// without (pair by pair: 2.0e-15).
 struct Cell64 {
   double vx, vy, vz;
-  double P0, K1, tt, L0, rt, d, rho;
+  double P0, K1, tt, L0, rt, d2, rho, r6, r24;
 };
 template <int M>
 __device__ __forceinline__ Cell64 cell64(const Mom64& m) {
@@ -226,7 +223,9 @@ __device__ __forceinline__ Cell64 cell64(const Mom64& m) {
   c.P0 = __fma_rn(c.rho, K0m1, m.r);
   c.K1 = __dmul_rn(c.rt, __fma_rn(t, -0.25 * (D + 2), __fma_rn(q, -0.25, 0.5)));
   c.L0 = __fma_rn(c.rt, -0.5 * (D + 2), __dmul_rn(c.rho, __fma_rn(q, -0.5, 1.0)));
-  c.d = __dsub_rn(c.L0, c.rt);
+  c.d2 = __dmul_rn(__dsub_rn(c.L0, c.rt), 0.5);
+  c.r6 = __dmul_rn(c.rho, 1.0 / 6.0);
+  c.r24 = __dmul_rn(c.rho, 1.0 / 24.0);
   return c;
 }
 
@@ -256,6 +255,11 @@ static __device__ __noinline__ Two64 relax_pair64(double ev, double od, double h
   return {fx_to<60>(p + fx_mul(v + o - p, om), e), fx_to<60>(m + fx_mul(v - o - m, om), e)};
 }
 
+template <int K>
+__device__ __forceinline__ double times64(double v) {
+  if constexpr (K == 1) return v; else return __dmul_rn((double)K, v);
+}
+
 // The relaxation h' = h + omega (h^eq - h) of one part's pairs.
 template <int M, int P, class Get, class Store>
 __device__ __forceinline__ void relax64(const Cell64& c, double omega, Get&& hv, Store&& st) {
@@ -272,11 +276,11 @@ __device__ __forceinline__ void relax64(const Cell64& c, double omega, Get&& hv,
     }
     // the shell's coefficients: the same expressions for each of its pairs, which the
     // compiler forms once
-    const double c0 = __fma_rn(mc.X4o8[g], c.tt, __fma_rn(mc.X2[g], c.K1, c.P0));
-    const double c1 = __fma_rn(mc.kX2o2[g], c.rt, __dmul_rn((double)k, c.L0));
-    const double c2 = __fma_rn(mc.k2X2o4[g], c.rt, __dmul_rn(0.5 * k * k, c.d));
-    const double c3 = __dmul_rn(k * k * k / 6.0, c.rho);
-    const double c4 = __dmul_rn(k * k * k * k / 24.0, c.rho);
+    const double c0 = __fma_rn(mc.X2[g], __fma_rn(mc.X2o8[g], c.tt, c.K1), c.P0);
+    const double c1 = times64<k>(__fma_rn(mc.X2o2[g], c.rt, c.L0));
+    const double c2 = times64<k * k>(__fma_rn(mc.X2o4[g], c.rt, c.d2));
+    const double c3 = times64<k * k * k>(c.r6);
+    const double c4 = times64<k * k * k * k>(c.r24);
     const double ev = __fma_rn(s2, __fma_rn(s2, c4, c2), c0);
     const double od = __dmul_rn(s, __fma_rn(s2, c3, c1));
     const double hp = hv(std::integral_constant<int, i>{});

@@ -23,10 +23,10 @@ struct ModelConst {
   float ef[kMaxQc][3]; // lattice vectors (loops that index directions at run time)
   // the FP64 form
   double W[kMaxGc], X2[kMaxGc];
+  double X2o2[kMaxGc], X2o4[kMaxGc], X2o8[kMaxGc];   // X2 / 2, / 4, / 8 (exact)
   double WX2[kMaxGc], WX4[kMaxGc];   // W X2, W X2^2
   // with k the gcd of the group's components (e = k b, b primitive):
   double Wk[kMaxGc], Wk2[kMaxGc], Wk3[kMaxGc], Wk4[kMaxGc];   // W k, W k^2, ...
-  double X4o8[kMaxGc], kX2o2[kMaxGc], k2X2o4[kMaxGc];   // X2^2 / 8, k X2 / 2, k^2 X2 / 4
   double a;            // sqrt(2) c: xi_i = a e_i
   double c;
   double T0;           // 1 / (2 c^2), lattice units

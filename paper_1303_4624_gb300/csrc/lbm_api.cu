@@ -200,6 +200,9 @@ bool build_host_model(int model, HostModel* hm) {
   for (int g = 0; g < G; ++g) {
     mc.W[g] = hm->W[g];
     mc.X2[g] = a * a * vs.e2[g];
+    mc.X2o2[g] = mc.X2[g] / 2.0;
+    mc.X2o4[g] = mc.X2[g] / 4.0;
+    mc.X2o8[g] = mc.X2[g] / 8.0;
     mc.WX2[g] = mc.W[g] * mc.X2[g];
     mc.WX4[g] = mc.WX2[g] * mc.X2[g];
     mc.Wf[g] = (float)mc.W[g];
@@ -217,9 +220,6 @@ bool build_host_model(int model, HostModel* hm) {
     mc.Wk2[g] = k * k * mc.W[g];
     mc.Wk3[g] = k * k * k * mc.W[g];
     mc.Wk4[g] = k * k * k * k * mc.W[g];
-    mc.X4o8[g] = mc.X2[g] * mc.X2[g] / 8.0;
-    mc.kX2o2[g] = k * mc.X2[g] / 2.0;
-    mc.k2X2o4[g] = k * k * mc.X2[g] / 4.0;
     mc.w[i] = hm->w[i];
     mc.iw[i] = 1.0 / hm->w[i];
     mc.iw2[i] = std::fma(-mc.iw[i], hm->w[i], 1.0) * mc.iw[i];

@@ -38,7 +38,7 @@ static inline double __fma_rn(double a, double b, double c) { return std::fma(a,
 namespace lbm {
 // What collide64.cuh reads of the model tables (common.h has the whole).
 struct ModelConst {
-  double W[10], X2[10], WX2[10], Wk[10], X4o8[10], kX2o2[10], k2X2o4[10], a;
+  double W[10], X2[10], X2o2[10], X2o4[10], X2o8[10], a;
 };
 static ModelConst c_mc[2];
 template <int I, int N, class F>
@@ -70,22 +70,24 @@ static void collide(double* h, double omega) {
 }
 
 extern "C" {
-void host_setup(int m, int Q, const double* w, const int* group, const int* e, double a) {
+void host_setup(int m, const double* w, double a) {
+  const auto& vs = m ? Model<1>::vs : Model<0>::vs;
   ModelConst& mc = c_mc[m];
   mc.a = a;
-  for (int i = 0; i < Q; ++i) {
-    const int g = group[i], *v = e + 3 * i;
-    const int k = igcd(igcd(iabs(v[0]), iabs(v[1])), iabs(v[2]));
+  for (int i = 0; i < vs.Q; ++i) {
+    const int g = vs.grp[i], *v = vs.e[i];
     mc.W[g] = w[i];
     mc.X2[g] = a * a * (v[0] * v[0] + v[1] * v[1] + v[2] * v[2]);
-    mc.WX2[g] = mc.W[g] * mc.X2[g];
-    mc.Wk[g] = k * mc.W[g];
-    mc.X4o8[g] = mc.X2[g] * mc.X2[g] / 8.0;
-    mc.kX2o2[g] = k * mc.X2[g] / 2.0;
-    mc.k2X2o4[g] = k * k * mc.X2[g] / 4.0;
+    mc.X2o2[g] = mc.X2[g] / 2.0;
+    mc.X2o4[g] = mc.X2[g] / 4.0;
+    mc.X2o8[g] = mc.X2[g] / 8.0;
   }
 }
-int host_group(int m, int i) { return m ? Model<1>::vs.grp[i] : Model<0>::vs.grp[i]; }
+// The lattice vectors in storage order, three components each.
+void host_velocities(int m, int* e) {
+  const auto& vs = m ? Model<1>::vs : Model<0>::vs;
+  for (int i = 0; i < 3 * vs.Q; ++i) e[i] = vs.e[i / 3][i % 3];
+}
 // One collision of each of n cells, h[cell][Q], in place.
 void host_collide(int m, double* h, long n, double omega) {
   for (long c = 0; c < n; ++c) m ? collide<1>(h + c * Model<1>::Q, omega) : collide<0>(h + c * Model<0>::Q, omega);
