@@ -231,11 +231,11 @@ __device__ __forceinline__ Cell64 cell64(const Mom64& m) {
 
 // h + omega (h^eq - h) of a pair's two members, h^eq = ev +- od: in fixed point at the
 // scale of the largest of the four terms (about 160 integer instructions for six at the FP64
-// rate); om is omega in units of 2^-62.  The error is at most nine units of 2^-60 of that
-// term's power of two (five from the terms' truncation, four from the product), without a
-// preferred sign, against omega 2^-53 of it in FP64; a smaller omega than 2^-6 (0 must
-// return h as it is) keeps the FP64 operations (tested on om: an FP64 comparison would cost
-// as much as an addition).
+// rate); om is omega in units of 2^-62.  The error is at most six units of 2^-60 of that
+// term's power of two (five from the terms' truncation, half a one from the product),
+// against omega 2^-53 of it in FP64; a smaller omega than 2^-6 (0 must return h as it is)
+// keeps the FP64 operations (tested on om: an FP64 comparison would cost as much as an
+// addition).
 struct Two64 {
   double p, m;
 };

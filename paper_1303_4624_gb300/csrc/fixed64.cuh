@@ -39,24 +39,24 @@ __device__ __forceinline__ double fx_to(long long i, int e) {
   const unsigned long long u = (unsigned long long)((i ^ s) - s);
   const int lz = __clzll((long long)u);
   const unsigned long long m = u << (lz & 63);
-  const unsigned low = (unsigned)m;
-  const unsigned up = ((low & 0x7ffu) + 0x3ffu + ((low >> 11) & 1u)) >> 11;
-  const unsigned long long f = (m >> 11) + up;                // 53 bits, rounded
+  const unsigned long long f0 = m >> 11;
+  const unsigned rest = ((unsigned)m << 21) | ((unsigned)f0 & 1u);
+  const unsigned long long f = f0 + (rest > 0x80000000u);     // 53 bits, rounded
   const int exponent = e + (63 - B) + 1 - lz;                 // field of the leading bit
   unsigned long long bits = ((unsigned long long)(unsigned)(exponent - 1) << 52) + f;
   bits |= (unsigned long long)s & 0x8000000000000000ull;
   return __longlong_as_double(u == 0 ? 0ll : (long long)bits);
 }
-// a f / 2^62 for |a| < 2^62 and an even factor f in [0, 2^63), |a f| < 2^125: three wide
-// products of the halves ah, al (a = 2^32 ah + 2 al + its lowest bit) and fh, fl.  Left out
-// are al fl, below four units, and the bits below a unit; `half` is their mean for this f
-// (al anywhere in its range) and ties go by al's last bit, so that the error, within four
-// units, has no preferred sign: a relaxation repeated at one omega would add it up.
+// a f / 2^62 to the nearest integer, for |a| < 2^62 and an even factor f in [0, 2^63) with
+// |a f| < 2^125: the wide products of the halves ah, al (a = 2^32 ah + 2 al + a0) and fh, fl.
+// A relaxation repeated at one omega adds up whatever its product leaves out or rounds one
+// way, so nothing is left out but bits below 2^-29 of a unit, and of two equally near
+// integers (omega = 1.5 has them often) al's last bit chooses.  0 gives 0.
 __device__ __forceinline__ long long fx_mul(long long a, long long f) {
   const int fh = (int)(f >> 32), fl = (int)((unsigned)f >> 1);
   const int ah = (int)(a >> 32), al = (int)((unsigned)a >> 1), a0 = (int)a & 1;
-  const int half = (1 << 28) + (fl >> 1) - (al & 1);
-  const long long t = (long long)ah * fl + ((long long)al * fh + ((long long)a0 * (fh >> 1) + half));
+  const unsigned low = (unsigned)(((long long)al * fl) >> 31) + (1u << 28) - (unsigned)(al & 1);
+  const long long t = (long long)ah * fl + ((long long)al * fh + (low + (unsigned)(a0 * (fh >> 1))));
   return (long long)ah * fh * 4 + (t >> 29);
 }
 

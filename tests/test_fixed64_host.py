@@ -66,21 +66,37 @@ def test_conversion_keeps_60_bits(host):
 
 
 @pytest.mark.parametrize("omega", [2.0 ** -6, 0.3, 1.0, 1.2, 1.5, 1.8, 1.999])
-def test_product_by_omega_has_no_preferred_sign(host, omega):
-    """Error within four units; its mean over n products within 6 standard deviations of 0 for
-    errors of at most 4 units each (4 / sqrt(n) is one)."""
+def test_product_by_omega_rounds_to_nearest(host, omega):
+    """Error at most half a unit and 2^-28 (two truncated terms below 2^-29 each), zero of zero
+    and of terms far below a unit; the mean error of n products within 6 standard deviations
+    of 0 for errors of at most half a unit each (0.5 / sqrt(n) is one)."""
     rng = np.random.default_rng(3)
     n, err = 20000, []
-    for _ in range(n):
-        a = int(rng.integers(-3 << 60, 3 << 60))
-        err.append(float(host.host_fx_mul(a, omega) - Fraction(a) * Fraction(omega)))
-    assert np.max(np.abs(err)) <= 4.0
-    assert abs(np.mean(err)) <= 6 * 4 / np.sqrt(n)
+    assert host.host_fx_mul(0, omega) == 0
+    for k in range(n):
+        a = int(rng.integers(-3 << 60, 3 << 60)) >> (k % 60 if k % 4 == 0 else 0)
+        err.append(Fraction(host.host_fx_mul(a, omega)) - Fraction(a) * Fraction(omega))
+    assert max(abs(v) for v in err) <= Fraction(1, 2) + Fraction(1, 1 << 28)
+    assert abs(float(sum(err)) / n) <= 6 * 0.5 / np.sqrt(n)
+
+
+@pytest.mark.parametrize("omega", [0.3, 1.0, 1.2, 1.5, 1.8, 1.999])
+def test_equilibrium_is_a_fixed_point(host, omega):
+    """A pair at its equilibrium stays there bit for bit, the rest state's zeros among them."""
+    rng = np.random.default_rng(5)
+    for k in range(500):
+        ev = 0.0 if k % 5 == 0 else float(rng.standard_normal() * 10.0 ** rng.uniform(-12, 0))
+        od = 0.0 if k % 3 == 0 else ev * float(rng.integers(-64, 65)) / 64.0
+        if Fraction(ev + od) != Fraction(ev) + Fraction(od) or Fraction(ev - od) != Fraction(ev) - Fraction(od):
+            continue
+        hp, hm = ctypes.c_double(ev + od), ctypes.c_double(ev - od)
+        host.host_relax(ev, od, ctypes.byref(hp), ctypes.byref(hm), omega)
+        assert (hp.value, hm.value) == (ev + od, ev - od)
 
 
 @pytest.mark.parametrize("omega", [2.0 ** -6, 1.0, 1.2, 1.8, 1.999])
 def test_relaxation_of_a_pair(host, omega):
-    """h + omega (h^eq - h) within nine units of 2^-60 of the largest term's power of two and
+    """h + omega (h^eq - h) within six units of 2^-60 of the largest term's power of two and
     one FP64 rounding, terms spread over 18 decades, zeros among them."""
     rng = np.random.default_rng(4)
     for _ in range(3000):
@@ -92,7 +108,7 @@ def test_relaxation_of_a_pair(host, omega):
         unit = Fraction(2) ** (int(np.frexp(np.abs(t).max())[1]) - 60)
         for got, h, eq in ((gp.value, hp, Fraction(ev) + Fraction(od)), (gm.value, hm, Fraction(ev) - Fraction(od))):
             want = Fraction(h) + Fraction(omega) * (eq - Fraction(h))
-            assert abs(Fraction(got) - want) <= 9 * unit + abs(want) * Fraction(2) ** -53
+            assert abs(Fraction(got) - want) <= 6 * unit + abs(want) * Fraction(2) ** -53
 
 
 def collide(e, w, a, D, h, omega):
