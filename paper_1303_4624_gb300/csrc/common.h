@@ -34,6 +34,7 @@ struct ModelConst {
   double w[kMaxQc];                 // weight
   double iw[kMaxQc], iw2[kMaxQc];   // 1 / w rounded, and the rest of it
   float iwf[kMaxQc], iwlo[kMaxQc];  // 1 / w as a double-float (hi, lo) pair
+  float iw2f[kMaxQc];               // iw2 rounded to FP32
   int e[kMaxQc][3];                 // lattice vectors (zero-padded to 3 components)
 };
 

@@ -1490,6 +1490,12 @@ template <class S>
 static __device__ __noinline__ S enc_any(double f, double w) {
   return Codec<S>::enc(f / w - 1.0);
 }
+// h = v / w - 1 of the FP64 form with d = v - w outside 2^-63 <= |d| < 2^64.
+static __device__ __noinline__ double set64_any(double v, double d, double iw, double iw2, double w) {
+  const int top = __double2hiint(d) & 0x7fffffff;
+  if ((top | __double2loint(d)) == 0) return 0.0;
+  return top < 0x3ff00000 ? __fma_rn(d, iw, __dmul_rn(d, iw2)) : v / w - 1.0;
+}
 // (double)v on the integer pipe (subnormals, Inf and NaN: the conversion instruction).
 __device__ __forceinline__ double widen(float v) {
   const unsigned u = __float_as_uint(v), m = u & 0x7fffffffu;
@@ -1504,7 +1510,7 @@ struct IoWeight {
   int i;
   long long next;            // first element of the next direction
   double w, iw, iw2;
-  float iwf, iwlo;
+  float iwf, iwlo, iw2f;
   __device__ __forceinline__ IoWeight(const ModelConst& mc, long long k, long long ncell) {
     i = (int)(k / ncell);
     next = (i + 1) * ncell;
@@ -1516,6 +1522,7 @@ struct IoWeight {
     iw2 = mc.iw2[i];
     iwf = mc.iwf[i];
     iwlo = mc.iwlo[i];
+    iw2f = mc.iw2f[i];
   }
   __device__ __forceinline__ void advance(const ModelConst& mc, long long k, long long ncell) {
     if (k < next) return;
@@ -1584,10 +1591,17 @@ __global__ void __launch_bounds__(kIoThreads)
   if (k >= n) return;
   auto one = [&](double v, const IoWeight& q) -> S {
     if constexpr (std::is_same<S, double>::value) {
-      // v / w - 1 with 1 / w = iw + iw2: half an ulp of 1, as the division and the
-      // subtraction had, in two FMAs (Inf and NaN as they are)
-      if ((__double2hiint(v) & 0x7ff00000) == 0x7ff00000) return v;
-      return __fma_rn(v, q.iw, __fma_rn(v, q.iw2, -1.0));
+      // d / w of d = v - w, exact where v is near w, with 1 / w = iw + iw2: one FMA at h's own
+      // size, to which d iw2 (an ulp of it at most) needs no more than FP32.  With the -1 last
+      // instead, or without iw2, every population of a direction is off the same way.
+      const double d = __dsub_rn(v, q.w);
+      const unsigned t = (unsigned)__double2hiint(d) & 0x7fffffffu, e = t >> 20;
+      if (e < 960u || e >= 1087u) return set64_any(v, d, q.iw, q.iw2, q.w);   // |d| < 2^-63, >= 2^64
+      const float dh = __uint_as_float(((unsigned)__double2hiint(d) & 0x80000000u) |
+                                       __funnelshift_l((unsigned)__double2loint(d), t - 0x38000000u, 3));
+      const unsigned c = __float_as_uint(__fmul_rn(dh, q.iw2f)), m = c & 0x7fffffffu;
+      const unsigned hi = m < 0x00800000u ? 0u : (c & 0x80000000u) | ((m >> 3) + 0x38000000u);
+      return __fma_rn(d, q.iw, __hiloint2double((int)hi, (int)(c << 29)));
     } else {
       const double d = __dsub_rn(v, q.w);
       FF s;
