@@ -1611,14 +1611,20 @@ __global__ void __launch_bounds__(kIoThreads)
       e = __fmaf_rn(s.hi, q.iwlo, e);
       e = __fmaf_rn(s.lo, q.iwf, e);
       const FF h = ff_renorm(p, e);
+      // Next to a midpoint of two stored values (within 2^-18 of half an ulp of hi, which
+      // covers the double-float error) the FP64 sequence decides the rounding.  hi is h rounded
+      // to FP32, so a 16-bit midpoint is near only where hi is that midpoint (the 13 or 16
+      // dropped bits 1000...) and lo is small.  FP32: also FP64's own 2^-53 of f / w, for |h|
+      // above 1e-3 (closer in proportion below), and at a power of two.
+      const unsigned u = __float_as_uint(h.hi);
+      const float half_ulp = __uint_as_float((u & 0x7f800000u) - (24u << 23));
       if constexpr (sizeof(S) == 4) {
-        // next to a midpoint of two FP32 values (within 2^-18 of half an ulp, which covers
-        // the double-float error and FP64's own 2^-53 of f / w for |h| above 1e-3; closer
-        // in proportion below), or at a power of two, the FP64 sequence decides the rounding
-        const unsigned u = __float_as_uint(h.hi);
-        const float half_ulp = __uint_as_float((u & 0x7f800000u) - (24u << 23));
         const float tol = __fmaf_rn(half_ulp, 0x1p-18f, 0x1p-52f * (1.0f + fabsf(h.hi)));
         if (h.hi != 0.f && (fabsf(fabsf(h.lo) - half_ulp) <= tol || (u & 0x007fffffu) == 0))
+          return enc_any<S>(v, q.w);
+      } else {
+        constexpr unsigned kDrop = std::is_same<S, __half>::value ? 0x1fffu : 0xffffu;
+        if ((u & kDrop) == (kDrop + 1) / 2 && fabsf(h.lo) <= half_ulp * 0x1p-18f)
           return enc_any<S>(v, q.w);
       }
       return ff_round<S>(h);
