@@ -10,8 +10,8 @@
 namespace lbm {
 
 // ----------------------------------------------------------------- adjoint
-// Discrete adjoint of one pull stream-collide step (exact transpose, arithmetic
-// type L = FP32 or FP64).  Variables are derivatives with respect to the
+// Discrete adjoint of one pull stream-collide step (exact transpose; k_adjoint in FP32 for
+// the FP32, FP16 and BF16 forms, k_adjoint64 for the FP64 form).  Variables are derivatives with respect to the
 // physical populations f.  With nu_n(x, j) = dL/dg^(n)_j(x) for the populations
 // gathered by step n and lambda_{n+1}(x, i) = dL/dS_{n+1}(x, i) = nu_{n+1}(x + e_i, i):
 //   nu_n(x, j) = (1 - omega) lambda_j + omega (alpha + beta . xi_j + gamma |xi_j|^2)
@@ -92,6 +92,7 @@ __global__ void __launch_bounds__(kAdjThreads, LBM_ADJ_MINB)
               double* __restrict__ omega_acc, Grid g, double omega) {
   using Mo = Model<M>;
   using Rt = L;
+  static_assert(std::is_same<L, float>::value, "the FP64 form has k_adjoint64");
   constexpr int D = Mo::D, RR = Mo::R, NP = Mo::NP;
   // the lambda copies are committed in kGroups groups of kPerGroup pairs; pass 1
   // waits for each group just before its first pair
@@ -185,9 +186,7 @@ __global__ void __launch_bounds__(kAdjThreads, LBM_ADJ_MINB)
     // the arithmetic type suffice here (they fix where the Jacobian is taken, to
     // ~1e-7 relative in FP32; the gradients are compared at 1e-4).
     const Rt rho_r = Rt(1) + rs;
-    Rt ir_r;
-    if constexpr (std::is_same<Rt, float>::value) ir_r = __fdividef(1.0f, rho_r);
-    else ir_r = 1.0 / rho_r;
+    const Rt ir_r = __fdividef(1.0f, rho_r);
     const double rho_d = (double)rho_r;
     const Rt ux = gA<Rt>(mc) * jx * ir_r;
     const Rt uy = gA<Rt>(mc) * jy * ir_r;
@@ -290,7 +289,8 @@ __global__ void __launch_bounds__(kAdjThreads, LBM_ADJ_MINB)
 // instructions counted (see collide64.cuh and contract.cuh): the forward moments shell by
 // shell, the contractions once per primitive vector; ~600 FP64 operations a D2Q33 cell
 // against ~900 pair by pair.  Linear cell index, 32 cells per block, shared by WARPS = 1, 2
-// or 4 warps as in k_stream_collide64.
+// or 4 warps as in k_stream_collide64; but a warp sums its own parts before the warps' sums
+// meet, so the last bits of a gradient depend on WARPS (the forward step's do not).
 template <int M, bool kFirst, int WARPS>
 __global__ void __launch_bounds__(32 * WARPS, 8 / WARPS)
     k_adjoint64(const double* __restrict__ state, const double* __restrict__ nu_next,

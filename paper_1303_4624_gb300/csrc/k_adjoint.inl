@@ -58,7 +58,7 @@ cudaError_t adjoint_m(const void* state_n, const void* nu_next, const double* dl
   const dim3 grid((unsigned)((g.nx + bx - 1) / bx), (unsigned)g.ny, (unsigned)g.nz);
   constexpr int smem = adj_smem_bytes<M, L>();
   const AdjointFn kern = dldrho ? adjoint_kernel<M, true>(g) : adjoint_kernel<M, false>(g);
-  if constexpr (smem > 0) {
+  {
     // Dynamic shared memory above the 48 KB default needs the opt-in, once per device.
     static std::mutex mu;
     static int done_dev[16] = {-1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1};

@@ -75,15 +75,6 @@ struct Codec<__nv_bfloat16> {
   }
   static __device__ __forceinline__ __nv_bfloat16 enc(double v) { return __double2bfloat16(v); }
 };
-template <class S>
-__device__ __forceinline__ double to_double(S v) {
-  if constexpr (std::is_same<S, __half>::value)
-    return (double)__half2float(v);
-  else if constexpr (std::is_same<S, __nv_bfloat16>::value)
-    return (double)__bfloat162float(v);
-  else
-    return (double)v;
-}
 
 // ----------------------------------------------------------------- helpers
 template <int I, int N, class F>
