@@ -20,8 +20,21 @@ AdjointFn adjoint_kernel(const Grid& g) {
   return k_adjoint<M, S, L, kFirst, false>;
 }
 
-// FP64 form: 32 cells per block, 1, 2 or 4 warps (lin64_warps: the adjoint step has about
-// three times the forward step's instructions in both of its terms).
+// FP64 form: warps per 32 cells, by the blocks of 32 cells an SM gets, as step64_warps.  All
+// measured (us an adjoint step with 1 / 2 / 4 warps, 152 SMs):
+//   D3Q95, blocks an SM 1: 61.9 / 41.2 / 35.0, 2: 66.8 / 51.1 / 53.7, 3: 65.2 / 54.6 / 60.3,
+//   5: 88.7 / 85.5 / 103, 6: 100 / 97 / 125, 7: 106 / 127 / 145, 8: 122 / 128 / 167,
+//   9: 186 / 156 / 184, 14: 247 / 220 / 283, 27: 453 / 429 / 532, 432: 6852 / 6542 / 8282
+//   D2Q33, 64 blocks: 25.6 / 16.5 / 14.0, 112: 26.6 / 17.2 / 15.4, 128: 25.8 / 17.3 / 18.3, an SM
+//   2: 25.6 / 20.7 / 25.2, 3: 28.6 / 25.0 / 32.7, 4: 30.3 / 31.9 / 42.1, 5: 38.7 / 41.4 / 53.2,
+//   14: 96 / 100 / 140, 432: 2475 / 2967 / 4258.
+template <int M>
+int adjoint64_warps(long long ncell, int sms) {
+  const long long all = (ncell + 31) / 32, blocks = (all + sms - 1) / sms;
+  if (M == 0) return 4 * all <= 3 * sms ? 4 : blocks <= 3 ? 2 : 1;
+  return blocks == 1 ? 4 : blocks == 7 || blocks == 8 ? 1 : 2;
+}
+
 template <int M>
 cudaError_t adjoint64_m(const void* state_n, const void* nu_next, const double* dldrho,
                         void* nu_out, double* omega_acc, const Grid& g, double omega,
@@ -29,7 +42,7 @@ cudaError_t adjoint64_m(const void* state_n, const void* nu_next, const double* 
   int sms = 0;
   cudaError_t e = sm_count(&sms);
   if (e != cudaSuccess) return e;
-  const int w = lin64_warps<M>(g.ncell, sms);
+  const int w = adjoint64_warps<M>(g.ncell, sms);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)((g.ncell + 31) / 32));
   cfg.blockDim = dim3(32 * w);

@@ -204,14 +204,14 @@ cudaError_t sm_count(int* sms) {
   return cudaSuccess;
 }
 
-// The FP64 kernel: 32 cells per block, 1, 2 or 4 warps (lin64_warps).
+// The FP64 kernel: 32 cells per block, 1, 2 or 4 warps (step64_warps; D3Q95 2 or 4).
 template <int M>
 cudaError_t step64_m(const void* src, void* dst, const Grid& g, double omega, int rev,
                      const Ends& ends, cudaStream_t st) {
   int sms = 0;
   cudaError_t e = sm_count(&sms);
   if (e != cudaSuccess) return e;
-  const int w = lin64_warps<M>(g.ncell, sms);
+  const int w = step64_warps<M>(g.ncell, sms);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)((g.ncell + 31) / 32));
   cfg.dynamicSmemBytes = Model<M>::Q * 32 * sizeof(double);
@@ -222,10 +222,10 @@ cudaError_t step64_m(const void* src, void* dst, const Grid& g, double omega, in
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  auto kern = k_stream_collide64<M, false, 1>;
-  if (w == 1) kern = rev ? k_stream_collide64<M, true, 1> : k_stream_collide64<M, false, 1>;
-  else if (w == 2) kern = k_stream_collide64<M, false, 2>;
-  else kern = k_stream_collide64<M, false, 4>;
+  auto kern = w == 2 ? k_stream_collide64<M, false, 2> : k_stream_collide64<M, false, 4>;
+  if constexpr (M == 0) {
+    if (w == 1) kern = rev ? k_stream_collide64<M, true, 1> : k_stream_collide64<M, false, 1>;
+  }
   return cudaLaunchKernelEx(&cfg, kern, static_cast<const double*>(src), static_cast<double*>(dst),
                             g, omega, ends);
 }

@@ -732,16 +732,16 @@ inline bool linear_rows(const Grid& g, int sms) {
 // FP64 form: linear cell index (rows of any length fill the warps), 32 cells per block,
 // WARPS warps per block.  The FP64 pipe bounds the form (see collide64.cuh): each of an
 // SM's four schedulers takes 64 cycles an FP64 instruction, so the grid's time is that of
-// the scheduler with the most warps.  Blocks of one warp spread them evenly (256 x 8
-// D2Q33: 64 warps on as many SMs, against 16 SMs with four each); where even so there are
-// fewer warps than schedulers, WARPS = 2 or 4 warps share 32 cells: each takes some of the
-// parts of collide64, and the parts' moments are exchanged through shared memory and
-// summed in collide64's order, so every WARPS gives the same bits (see lin64_warps for
-// the rule).
+// the scheduler with the most work.  Small blocks spread it evenly (256 x 8 D2Q33: 64 of them
+// on as many SMs), and with WARPS = 2 or 4 warps sharing 32 cells more schedulers work and
+// each has more warps to choose from (a warp alone waits for its FP64 results): every warp
+// takes some of the parts of collide64, and the parts' moments are exchanged through shared
+// memory and summed in collide64's order, so every WARPS gives the same bits (see
+// step64_warps for the rule).
 // Each thread copies its populations to shared memory first (cp.async, its own copies only,
 // so no barrier): they are used twice, for the moments and for the relaxation, 95 doubles
 // would take 190 registers, and read again from L1 / L2 they stall the few warps an SM
-// holds (D3Q95 128 x 32 x 32: 190 us against 152).  24 KB a warp for D3Q95.
+// holds (D3Q95 128 x 32 x 32, one warp: 190 us against 152).  24 KB a block for D3Q95.
 template <int M, bool REV, int WARPS>
 __global__ void __launch_bounds__(32 * WARPS, 8 / WARPS)
     k_stream_collide64(const double* __restrict__ src, double* __restrict__ dst, Grid g,
@@ -830,24 +830,21 @@ __global__ void __launch_bounds__(32 * WARPS, 8 / WARPS)
   }
 }
 
-// Warps per 32 cells: the choice with the least work on the busiest
-// scheduler, ceil(warps / schedulers) times the time of a warp.  In units of an FP64
-// instruction that is about 170 / 580 for all pairs of D2Q33 / D3Q95 and 70 for what every
-// warp repeats (moment totals, 1 / rho, the coefficients of the cell).
+// Warps per 32 cells, by the blocks of 32 cells an SM gets.  All measured, 2k to 2M cells (us
+// a step with 1 / 2 / 4 warps, 152 SMs):
+//   D3Q95, blocks an SM 1: 35.1 / 18.7 / 13.2, 2: 35.4 / 19.6 / 17.8, 3: 35.6 / 23.6 / 33.3,
+//   4: 36.7 / 25.7 / 28.2, 5: 53.9 / 42.6 / 34.2, 6: 53.4 / 42.7 / 47.6, 8: 54.9 / 42.9 / 61.4,
+//   14: 86.9 / 74.7 / 102.8, 27: 155 / 148 / 200, 432: 2275 / 2248 / 3156
+//   (two warps a block fill the four schedulers evenly at 2, 4, 6, 8 blocks; at 5 three of
+//   them hold three warps, where four shorter warps a block balance better)
+//   D2Q33, 1: 14.1 / 9.1 / 7.3, 2: 14.3 / 9.7 / 10.4, 3: 14.4 / 11.8 / 13.4, 4: 14.8 / 13.3 /
+//   22.9, 5: 17.7 / 16.8 / 23.1, 6: 18.2 / 27.2 / 23.2, 7: 19.2 / 27.3 / 26.4, 14: 34.9 / 37.0 /
+//   49.2, 432: 833 / 991 / 1410.
 template <int M>
-inline int lin64_warps(long long ncell, int sms) {
-  const long long groups = (ncell + 31) / 32;
-  int best = 1;
-  long long best_cost = -1;
-  for (int w = 1; w <= 4; w *= 2) {
-    const long long rounds = (groups * w + 4LL * sms - 1) / (4LL * sms);
-    const long long cost = rounds * ((M == 0 ? 170 : 580) / w + 70);
-    if (best_cost < 0 || cost < best_cost) {
-      best = w;
-      best_cost = cost;
-    }
-  }
-  return best;
+inline int step64_warps(long long ncell, int sms) {
+  const long long blocks = ((ncell + 31) / 32 + sms - 1) / sms;
+  if (M == 0) return blocks == 1 ? 4 : blocks <= 5 ? 2 : 1;
+  return blocks <= 2 || blocks == 5 ? 4 : 2;
 }
 
 // ----------------------------------------------------------------- split kernel
