@@ -4,13 +4,15 @@
 // pipes take one every cycle or two: an FP64 addition costs as much as some fifty integer
 // instructions.  A group of doubles (the populations of a shell, or the terms of one
 // relaxation) is brought to a common exponent, that of its largest member, and added as
-// 64-bit integers.  With 56 or more bits below the largest member nothing is lost against
-// FP64's 53; integer sums do not depend on their order.
+// 64-bit integers, with B = 56 or 60 bits below that exponent: a member within 2^-3 (2^-7) of
+// the largest keeps its 53 bits, a smaller one loses less than 2^-B of that power of two,
+// where an FP64 sum rounds every partial sum at 2^-53 of itself.  Integer sums do not depend
+// on their order.
 //
 // top: the largest (high word & 0x7fffffff) of the group; its exponent field e bounds
 // |v| < 2^(e - 1022).  A value v is held as trunc(v 2^(B - (e - 1022))) with B bits.
 // Groups with an exponent field of 2000 or more (|v| >= 2^977, Inf, NaN) are the caller's
-// (fx_regular); fields below 64 count as 64 (|v| < 2^-1014 is held as 0).
+// (fx_regular: the moments of such a cell are NaN); fields below 64 count as 64 (|v| < 2^-1014 is held as 0).
 #pragma once
 
 namespace lbm {

@@ -928,11 +928,11 @@ __global__ void __launch_bounds__(kSplitThreads, LBM_SPLIT_MINB)
 // ----------------------------------------------------------------- equilibrium init
 // h_i = rho P_i(u, theta) - 1 for the fields rho, U (lattice), T (lattice) of each cell,
 // rounded once to the storage type.  FP64 for the FP64 form; double-float on the FP32
-// pipe for the FP32, FP16 and BF16 forms, whose ~48 significant bits round to the
-// same value as FP64 except within 2^-44 relative of a rounding boundary.  The five
-// FP64 inputs are split into double-float once and everything else runs on the FP32
-// pipe: on this GPU the FP64 pipe issues 1/64 of the FP32 rate, and the FP64 form of
-// the 95 direction polynomials is bound by it (~38 ms for 33.5 M cells; with the
+// pipe for the FP32, FP16 and BF16 forms, whose ~48 significant bits (~46 in the 16-bit
+// forms) round to the same value as FP64 except within 2^-44 (2^-42) relative of a rounding
+// boundary.  The five FP64 inputs are split into double-float once and everything else runs
+// on the FP32 pipe: on this GPU the FP64 pipe issues 1/64 of the FP32 rate, and the FP64
+// form of the 95 direction polynomials is bound by it (~38 ms for 33.5 M cells; with the
 // shell coefficients alone in FP64, ~13 ms; all in double-float, 6.7 ms).
 
 // double-float helpers (FMA products, Knuth / Dekker sums; see ff_add)
@@ -1101,7 +1101,8 @@ __global__ void __launch_bounds__(256)
       // 16-bit forms: the pairs of a primitive direction share s and s^2, rho is folded into
       // the shells' coefficients and the sums are not renormalised in between: 5000
       // instructions a D3Q95 cell against 6800 (8.2 -> 6.4 ms for 512 x 256 x 256, bound by
-      // issue), with ~46 significant bits before the one rounding.  The FP32 form, where that
+      // issue), with ~46 significant bits before the one rounding (states of 1.6e9
+      // values, flows, near rest and with jumps: bit for bit those of the renormalised sums).  The FP32 form, where that
       // would round about one result in 2^20 the other way, keeps the renormalised sums.
       // EqCoef's coefficients times rho
       const FF P0 = ff_add(rm1, ff_mul(r, K0m1)), rK1 = ff_mul(r, K1), rK2 = ff_mul(r, K2);
