@@ -1101,9 +1101,10 @@ __global__ void __launch_bounds__(256)
       // 16-bit forms: the pairs of a primitive direction share s and s^2, rho is folded into
       // the shells' coefficients and the sums are not renormalised in between: 5000
       // instructions a D3Q95 cell against 6800 (8.2 -> 6.4 ms for 512 x 256 x 256, bound by
-      // issue), with ~46 significant bits before the one rounding (states of 1.6e9
-      // values, flows, near rest and with jumps: bit for bit those of the renormalised sums).  The FP32 form, where that
-      // would round about one result in 2^20 the other way, keeps the renormalised sums.
+      // issue), with ~46 significant bits before the one rounding (states of 1.6e9 values,
+      // flows, near rest and with jumps: bit for bit those of the renormalised sums).  The FP32
+      // form, where that would round about one result in 2^20 the other way, keeps the
+      // renormalised sums.
       // EqCoef's coefficients times rho
       const FF P0 = ff_add(rm1, ff_mul(r, K0m1)), rK1 = ff_mul(r, K1), rK2 = ff_mul(r, K2);
       const FF rL0 = ff_mul(r, L0), rL1 = ff_mul(r, L1), rM0 = ff_mul(r, M0), rM1 = ff_mul(r, M1);
