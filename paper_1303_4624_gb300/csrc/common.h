@@ -10,7 +10,10 @@ namespace lbm {
 constexpr int kMaxQc = 95;
 constexpr int kMaxGc = 10;
 
-// Per-model constants solved on the host (Formula 5) and kept in constant memory.
+// Per-model constants solved on the host (Formula 5) and kept in constant memory, one table
+// for each model.  The size of the first decides how the second one's hot constants lie in the
+// constant cache's lines: 380 bytes more (at the end) cost the D3Q95 FP32 step 2.4 %
+// (512x256x256, 10 steps with init 50.3 -> 51.5 ms), so time that case after a change here.
 struct ModelConst {
   // read by the FP32-arithmetic kernels
   float Wf[kMaxGc];    // weight of each symmetry group
@@ -34,7 +37,6 @@ struct ModelConst {
   double w[kMaxQc];                 // weight
   double iw[kMaxQc], iw2[kMaxQc];   // 1 / w rounded, and the rest of it
   float iwf[kMaxQc], iwlo[kMaxQc];  // 1 / w as a double-float (hi, lo) pair
-  float iw2f[kMaxQc];               // iw2 rounded to FP32
   int e[kMaxQc][3];                 // lattice vectors (zero-padded to 3 components)
 };
 

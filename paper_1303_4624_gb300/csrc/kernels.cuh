@@ -1512,7 +1512,7 @@ struct IoWeight {
     iw2 = mc.iw2[i];
     iwf = mc.iwf[i];
     iwlo = mc.iwlo[i];
-    iw2f = mc.iw2f[i];
+    iw2f = (float)iw2;
   }
   __device__ __forceinline__ void advance(const ModelConst& mc, long long k, long long ncell) {
     if (k < next) return;

@@ -223,7 +223,6 @@ bool build_host_model(int model, HostModel* hm) {
     mc.w[i] = hm->w[i];
     mc.iw[i] = 1.0 / hm->w[i];
     mc.iw2[i] = std::fma(-mc.iw[i], hm->w[i], 1.0) * mc.iw[i];
-    mc.iw2f[i] = (float)mc.iw2[i];
     mc.iwf[i] = (float)mc.iw[i];
     mc.iwlo[i] = (float)(mc.iw[i] - (double)mc.iwf[i]);
     for (int d = 0; d < 3; ++d) {
