@@ -1369,8 +1369,7 @@ __device__ __forceinline__ void moments_fp64_form(const double* __restrict__ src
     double U2 = __fma_rn(Ux, Ux, __dmul_rn(Uy, Uy));
     if constexpr (D == 3) U2 = __fma_rn(Uz, Uz, U2);
     // T = T0 + ((E - D rho) T0 / rho - |U|^2) / D
-    const double t = __dmul_rn(
-        __fma_rn(mc.T0, over_rho(__fma_rn(-(double)D, m.r, m.e)), -U2), 1.0 / D);
+    const double t = over_dim64<D>(__fma_rn(mc.T0, over_rho(__fma_rn(-(double)D, m.r, m.e)), -U2));
     if (rho_out) rho_out[idx] = rho;
     if (U_out) {
       U_out[idx] = Ux;

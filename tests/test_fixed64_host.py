@@ -140,21 +140,28 @@ def collide(e, w, a, D, h, omega):
     return out
 
 
+def set_up(host, model):
+    """Lattice vectors in the library's order, their weights, a and D; the host tables filled."""
+    mdl, m = get_model(model), int(model == "D3Q95")
+    a = float(np.sqrt(2.0) * mdl.c)
+    order = np.zeros((mdl.Q, 3), np.int32)
+    host.host_velocities(m, order.ctypes.data_as(ctypes.c_void_p))
+    e = order[:, :mdl.D]
+    pos = {tuple(v): i for i, v in enumerate(mdl.e.tolist())}
+    w = np.ascontiguousarray([mdl.w[pos[tuple(v)]] for v in e.tolist()])
+    host.host_setup(m, w.ctypes.data_as(ctypes.c_void_p), ctypes.c_double(a))
+    return e, w, a, mdl.D
+
+
 @pytest.mark.parametrize("model,dims,steps,omega", [("D2Q33", (64, 8, 1), 150, 1.5), ("D2Q33", (25, 13, 1), 60, 1.2),
                                                     ("D3Q95", (16, 7, 6), 40, 1.8), ("D3Q95", (9, 8, 5), 40, 1.2)])
 def test_whole_runs_stay_as_near_to_exact_as_plain_fp64(host, model, dims, steps, omega):
     """A perturbed two-state flow: the populations' rms distance from extended precision after
     all steps is at most that of the same collision evaluated direction by direction in FP64,
     with a fifth for the scatter of two rounding sequences."""
-    mdl, m = get_model(model), int(model == "D3Q95")
-    D, Q = mdl.D, mdl.Q
-    a = float(np.sqrt(2.0) * mdl.c)
-    order = np.zeros((Q, 3), np.int32)
-    host.host_velocities(m, order.ctypes.data_as(ctypes.c_void_p))
-    pos = {tuple(v): i for i, v in enumerate(mdl.e.tolist())}
-    w = np.ascontiguousarray([mdl.w[pos[tuple(int(x) for x in v[:D])] if D == 2 else pos[tuple(int(x) for x in v)]]
-                              for v in order])
-    host.host_setup(m, w.ctypes.data_as(ctypes.c_void_p), ctypes.c_double(a))
+    m, (order, w, a, D) = int(model == "D3Q95"), set_up(host, model)
+    order = np.pad(order, ((0, 0), (0, 3 - D)))
+    Q = len(order)
     e = order.astype(np.float64)
     rng = np.random.default_rng(9)
     z, y, x = np.meshgrid(*[np.arange(n) for n in dims[::-1]], indexing="ij")
@@ -180,3 +187,23 @@ def test_whole_runs_stay_as_near_to_exact_as_plain_fp64(host, model, dims, steps
     got = run(h0, kernels)
     rms = lambda v: float(np.sqrt(np.mean((v - exact) ** 2)))
     assert rms(got) <= 1.2 * rms(plain)
+
+
+@pytest.mark.parametrize("model", ["D2Q33", "D3Q95"])
+def test_collision_has_no_bias(host, model):
+    """One collision of random near-equilibrium cells: each direction's mean error against
+    extended precision is within 6 standard deviations of its own mean of zero (every constant
+    that is multiplied in by a rounded value would show here)."""
+    m, (e, w, a, D) = int(model == "D3Q95"), set_up(host, model)
+    rng = np.random.default_rng(12)
+    n = 40000
+    r, t, u = rng.uniform(-0.4, 0.4, n), rng.uniform(-0.3, 0.3, n), 0.1 * rng.standard_normal((D, n))
+    h = np.empty((len(e), n))
+    for i in range(len(e)):
+        s, x, q = a * (e[i].astype(float) @ u), a * a * float(e[i] @ e[i]), (u * u).sum(0)
+        h[i] = r + (1 + r) * (-q / 2 + t * (x - D) / 2 + s * (1 + s / 2))
+    h *= 1 + 0.05 * rng.standard_normal(h.shape)
+    c = np.ascontiguousarray(h.T)
+    host.host_collide(m, c.ctypes.data_as(ctypes.c_void_p), ctypes.c_long(n), ctypes.c_double(1.0))
+    err = c.T - collide(e, w, a, D, h.astype(np.longdouble), 1.0)
+    assert np.all(np.abs(err.mean(axis=1)) <= 6 * err.std(axis=1) / np.sqrt(n))
