@@ -5,7 +5,8 @@
 // instruction, whatever the number of active lanes (measured, dependent or not; a
 // conversion between FP64 and FP32 costs the same), so the form is bound by its FP64
 // instruction count and not by memory: 1520 bytes a D3Q95 cell take 0.23 ns of HBM time,
-// the ~1290 FP64 operations of the pair-by-pair form 2.4 ns.  What brings D3Q95 to ~420:
+// the ~1290 FP64 operations of the pair-by-pair form 2.4 ns.  What brings D3Q95 to ~470 with
+// two warps sharing 32 cells (of which one repeats ~35):
 //   * moments shell by shell: the members of a shell share weight and |xi|^2, so their
 //     sums are formed unweighted and each shell is weighted once;
 //   * those sums, and the relaxation's h + omega (h^eq - h), in 64-bit fixed point on the
@@ -17,7 +18,7 @@
 //     coefficients.
 // Measured (us a step): D3Q95 128x32x32 311 pair by pair, 235 regrouped in FP64, 149 with
 // the fixed point; D2Q33 1024x512 446, 354, 210.
-// Error: runs of 40 to 150 steps end 0.2 to 0.5 as far from extended precision as the same
+// Error: runs of 40 to 150 steps end 0.2 to 0.45 as far from extended precision as the same
 // collisions evaluated direction by direction in FP64.
 //
 // The shells are dealt into kParts64 parts of nearly equal work (whole shells, so the
